@@ -36,7 +36,14 @@ extern "C" {
 #define MPFC_ERR_DIVERGED (-5)      /* residual became non-finite or grew by > 1e10     */
 #define MPFC_ERR_TOO_LARGE (-6)     /* grid larger than mpfc_mass_noalloc's static scratch allows */
 
-#define MPFC_FP64 0       /* every V-cycle kernel in FP64                                  */
+/* MPFC_FP64: FP64 iterate, source, residual, convergence test and state.  The V-cycle works on
+ * the change it makes to the iterate (correction form of the FAS cycle: the same iterates in
+ * exact arithmetic), carried in float-float numbers (48 bits) from an FP64 residual; a change
+ * of relative error 2^-46 leaves the converged step at the FP64 rounding level.  Values outside
+ * the range that form covers (|phi| >= 2^20, a residual >= 2^40 or below 2^-56 and still above
+ * tol) continue with FP64 V-cycles, and handles with a single level or stencil coefficients
+ * outside [2^-60, 2^60] (h far below 1e-4) use those alone. */
+#define MPFC_FP64 0
 #define MPFC_FP32_INNER 1 /* FP64 outer defect correction around FP32 inner V-cycles       */
 
 #define MPFC_LAUNCH_GRAPH 0  /* a time step is one CUDA graph with a device-side loop (default) */
@@ -204,14 +211,14 @@ int mpfc_fp32_test_withhold_copy(int withhold, long long spin_cycles);
  * depend on it).  Launches of at least small_cells cells use blocks of 32 x rows
  * threads (rows 1, 2, 4 or 8), smaller ones one-warp blocks; grids of at most
  * pdl_blocks blocks are launched with programmatic dependent launch (0: none).  The
- * V-cycle's levels of at most tail_cells cells (0: none) run as one launch: for the
- * FP64 path of one CTA (tail_ctas 1) or of a thread-block cluster of tail_ctas CTAs (8,
- * or 16 where the GPU can hold such a cluster), for the FP32 inner cycles of one CTA
- * with the levels in shared memory.  Drops the handle's captured graphs (rebuilt on the
+ * V-cycle's levels of at most tail_cells cells (0: none) run as one launch of one CTA
+ * with the levels in shared memory (as far as they fit); FP64 V-cycles outside the
+ * correction form (see MPFC_FP64) take one CTA (tail_ctas 1) or a thread-block cluster of
+ * tail_ctas CTAs (8, or 16 where the GPU can hold such a cluster).  Drops the handle's captured graphs (rebuilt on the
  * next step).  Returns MPFC_ERR_INVALID for other values. */
 int mpfc_set_launch_shape(mpfc_t* h, int rows, int small_cells, int pdl_blocks, int tail_cells, int tail_ctas);
 
-/* Thread layout of the FP64 V-cycle's grid transfers (App. B: the FAS restriction of u and
+/* Thread layout of the grid transfers of FP64 V-cycles outside the correction form (App. B: the FAS restriction of u and
  * of the residual, and the bilinear prolongation of the correction; a tuning choice:
  * results do not depend on it, bit for bit).  Onto or from fine levels of at most
  * fine_cells cells that run as per-level launches, the restriction takes four threads per

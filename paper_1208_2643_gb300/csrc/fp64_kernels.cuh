@@ -492,6 +492,47 @@ __device__ __forceinline__ void gauss_jordan_cols(float (&a)[R], int G, float* x
   __syncwarp();
 }
 
+// Gaussian elimination with row swaps of the G x (G + 1) augmented system A in shared
+// memory (last column the right-hand side), solution in d; one warp.
+__device__ __forceinline__ void gauss_shared(float* Jm, float* d, int G) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, W = G + 1;
+  for (int col = 0; col < G; ++col) {
+    float best = -1.f;
+    int piv = col;
+    for (int r = col + lane; r < G; r += 32) {
+      float v = fabsf(Jm[r * W + col]);
+      if (v > best) { best = v; piv = r; }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      float ob = __shfl_down_sync(FULL, best, o);
+      int op = __shfl_down_sync(FULL, piv, o);
+      if (ob > best || (ob == best && op < piv)) { best = ob; piv = op; }
+    }
+    piv = __shfl_sync(FULL, piv, 0);
+    if (piv != col)
+      for (int c2 = col + lane; c2 <= G; c2 += 32) {
+        float t = Jm[col * W + c2];
+        Jm[col * W + c2] = Jm[piv * W + c2];
+        Jm[piv * W + c2] = t;
+      }
+    __syncwarp();
+    float rp = 1.f / Jm[col * W + col];
+    for (int r = col + 1 + lane; r < G; r += 32) {
+      float f = Jm[r * W + col] * rp;
+      for (int c2 = col + 1; c2 <= G; ++c2) Jm[r * W + c2] = fmaf(-f, Jm[col * W + c2], Jm[r * W + c2]);
+    }
+    __syncwarp();
+  }
+  for (int r = G - 1; r >= 0; --r) {
+    float acc = 0.f;
+    for (int c2 = r + 1 + lane; c2 < G; c2 += 32) acc = fmaf(Jm[r * W + c2], d[c2], acc);
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(FULL, acc, o);
+    if (lane == 0) d[r] = (Jm[r * W + G] - acc) / Jm[r * W + r];
+    __syncwarp();
+  }
+}
+
 // The Newton iteration on the coarsest grid.  R > 0: grids of at most min(R, 31)
 // cells, one Jacobian column per lane in R registers (gauss_jordan_cols); R == 0:
 // up to 64 cells, Gaussian elimination with row swaps in shared memory.
@@ -611,40 +652,7 @@ __device__ void coarse_newton(const Lev& C, const Coef& k, const float* __restri
         Jm[r * W + col] = K3f[idx] - cLf[idx] * d[col];
       }
       __syncwarp();
-      for (int col = 0; col < G; ++col) {
-        float best = -1.f;
-        int piv = col;
-        for (int r = col + lane; r < G; r += 32) {
-          float v = fabsf(Jm[r * W + col]);
-          if (v > best) { best = v; piv = r; }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          float ob = __shfl_down_sync(FULL, best, o);
-          int op = __shfl_down_sync(FULL, piv, o);
-          if (ob > best || (ob == best && op < piv)) { best = ob; piv = op; }
-        }
-        piv = __shfl_sync(FULL, piv, 0);
-        if (piv != col)
-          for (int c2 = col + lane; c2 <= G; c2 += 32) {
-            float t = Jm[col * W + c2];
-            Jm[col * W + c2] = Jm[piv * W + c2];
-            Jm[piv * W + c2] = t;
-          }
-        __syncwarp();
-        float rp = 1.f / Jm[col * W + col];
-        for (int r = col + 1 + lane; r < G; r += 32) {
-          float f = Jm[r * W + col] * rp;
-          for (int c2 = col + 1; c2 <= G; ++c2) Jm[r * W + c2] = fmaf(-f, Jm[col * W + c2], Jm[r * W + c2]);
-        }
-        __syncwarp();
-      }
-      for (int r = G - 1; r >= 0; --r) {
-        float acc = 0.f;
-        for (int c2 = r + 1 + lane; c2 < G; c2 += 32) acc = fmaf(Jm[r * W + c2], d[c2], acc);
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(FULL, acc, o);
-        if (lane == 0) d[r] = (Jm[r * W + G] - acc) / Jm[r * W + r];
-        __syncwarp();
-      }
+      gauss_shared(Jm, d, G);
     }
     float dmax = 0.f;
     double umax = 0.0;
@@ -761,8 +769,7 @@ __device__ __forceinline__ bool grid_sum(double (&v)[NS], double* partials, unsi
 
 // The V-cycle loop decision from the scaled residual norm res (one thread).
 // mode 0: after the initial guess (sets res0); mode 1: after a V-cycle.
-__device__ __forceinline__ void resnorm_decide(Ctl* ctl, double res, int mode, cudaGraphConditionalHandle hnd,
-                                               int set_cond) {
+__device__ __forceinline__ bool resnorm_next(Ctl* ctl, double res, int mode) {
   int cond;
   if (mode == 0) {
     ctl->res0 = res;
@@ -778,7 +785,12 @@ __device__ __forceinline__ void resnorm_decide(Ctl* ctl, double res, int mode, c
   else if (ctl->fixed_cycles > 0) cond = ctl->cycles < ctl->fixed_cycles;
   else cond = (res > ctl->tol) && (ctl->cycles < ctl->max_cycles);
   if (mode == 0 && (!(res == res) || isinf(res))) { ctl->status = 2; cond = 0; }
-  if (set_cond) cudaGraphSetConditional(hnd, cond ? 1u : 0u);
+  return cond != 0;
+}
+__device__ __forceinline__ void resnorm_decide(Ctl* ctl, double res, int mode, cudaGraphConditionalHandle hnd,
+                                               int set_cond) {
+  const bool go = resnorm_next(ctl, res, mode);
+  if (set_cond) cudaGraphSetConditional(hnd, go ? 1u : 0u);
 }
 
 // Row 1 of the residual alone, r1 = S1 - phi + c Delta_h mu (as in resid_at).
@@ -847,6 +859,7 @@ static __global__ void k_step_begin(Ctl* ctl) {
     ctl->skip = ctl->halt;
     ctl->cycles = 0;
     ctl->status = 0;
+    ctl->range = 0;
   }
 }
 

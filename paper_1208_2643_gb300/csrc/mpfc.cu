@@ -244,6 +244,7 @@ static size_t carve(mpfc_s* H, const mpfc_params* p, char* base) {
   float* K3a = c.take<float>(2 * (size_t)Gc * Gc);   // K3 and c L of scheme 1 (mpfc_coarse_block)
   float* K3b = c.take<float>(2 * (size_t)Gc * Gc);
   mpfc_fp32_carve(H, p, &c.off, base, L);
+  mpfc_df_carve(H, p, &c.off, base, lev, px, pf, L);
   mpfc_guess_carve(H, p, &c.off, base);
   if (H && base) {
     H->nlev = L;
@@ -306,31 +307,25 @@ void mpfc_build_K3(const Lev& C, const Coef& k, std::vector<double>& K3) {
       K3[(size_t)r * G + c2] = (r == c2 ? 1.0 : 0.0) - k.c * k.theta * L3[(size_t)r * G + c2];
 }
 
-// Default launch shapes, from interleaved timings on GB300 (V-cycle at 1024^2):
-//   FP64: one-warp blocks everywhere and programmatic launch only for grids of at most
-//     16 blocks (the coarse tail, the coarsest levels' one-warp launches): 341 steps/s
-//     at 1024^2 (scheme 1) against 328 with programmatic launch up to 4 x SMs blocks and
-//     315 for every grid; 756 against 689 at 512^2, 662 against 613 for scheme 2 at
-//     512^2, 111 against 109 at 2048^2; only grids of about 128^2 gain from it (1466
-//     against 1501 steps/s there).  (An earlier driver favoured 4 x SMs: 743 against
-//     822 us per V-cycle with 32 x 8 blocks and none.)
-//   FP32 inner cycles (memory-latency bound, they want occupancy): 32 x 4 blocks and the
-//     same programmatic launch, 472 us per outer iteration against 479 (32 x 8, none)
-//     and 725 with one-warp blocks;
-//   the FP64 levels of at most 16 x 16 cells as one single-CTA launch: 701 us per
-//     V-cycle at 1024^2 against 721 without (a 16-CTA cluster: 719; at 64^2: 138, 162,
-//     155); larger tails were slower, their phases being bound by the FP64 instruction
-//     latency of the cell updates, not by launches;
-//   the FP32 inner cycles' levels of at most 32 x 32 cells in one CTA with the levels in
-//     shared memory: 430 us per outer iteration at 1024^2 against 475 (64 x 64: 457).
+// Default launch shapes, from interleaved timings on GB300:
+//   FP32 inner cycles (memory-latency bound, they want occupancy): 32 x 4 blocks and
+//     programmatic launch up to 4 x SMs blocks, 472 us per outer iteration at 1024^2
+//     against 479 (32 x 8, none) and 725 with one-warp blocks; the levels of at most
+//     32 x 32 cells in one CTA with the levels in shared memory: 430 us against 475
+//     (64 x 64: 457);
+//   FP64 handles, whose V-cycles run in correction form (float-float, bound by FP32 issue
+//     and memory): 32 x 4 blocks and programmatic launch up to 4 x SMs blocks, two steps at
+//     1024^2 in 3.62 ms against 4.24 (one-warp blocks), 3.67 (32 x 2) and 3.75 (32 x 8),
+//     one step at 4096^2 in 16.9 ms against 22.4, 17.1 and 17.3; programmatic launch for
+//     every grid costs 3 % at 4096^2.  The levels of at most 16 x 16 cells as one
+//     single-CTA launch (32 x 32: 3.60 ms at 1024^2; 64 x 64: 3.96).
+//   The FP64 V-cycle (outside the correction form's range only) prefers one-warp blocks and
+//     programmatic launch up to 128 blocks: 2.92 against 3.7 ms per step at 1024^2.
 mpfc_launch_shape mpfc_default_launch_shape(int precision) {
   if (precision == MPFC_FP32_INNER) return mpfc_launch_shape{4, 0, 4 * mpfc::sm_count(), 32 * 32, 1, 0};
-  // split transfers up to 256^2 fine cells: 2.917 against 2.975 ms per step at 1024^2
-  // (0: 2.975, 64^2: 2.934, 128^2: 2.920, 512^2: 2.962, 1024^2: 3.160); with them,
-  // programmatic launch up to 128 blocks (the split kernels' grids on levels up to 64^2):
-  // 2.916 against 2.926 ms with 16 blocks, 3.003 with 256 (the 128^2 sweeps), and 1.853
-  // against 1.864 ms for scheme 2 at 512^2; tails from 8^2 and 32^2 stay slower
-  return mpfc_launch_shape{1, 0, 128, 256, 1, 256 * 256};
+  // split transfers of the FP64 V-cycle up to 256^2 fine cells: 2.917 against 2.975 ms per
+  // step at 1024^2 without, with one-warp blocks
+  return mpfc_launch_shape{4, 0, 4 * mpfc::sm_count(), 256, 1, 256 * 256};
 }
 
 // The coarsest grid's matrices for one scheme as the FP32 block the coarse solves read:
@@ -373,6 +368,7 @@ extern "C" int mpfc_create(const mpfc_params* p, void* d_workspace, size_t bytes
       H->coef[s][l] = mpfc_coef(p, s + 1, H->lev[l].h, 4);
       H->coefb[s][l] = mpfc_coef(p, s + 1, H->lev[l].h, 3);
     }
+  H->df = mpfc_df_usable(H);
   int rc = MPFC_OK;
   do {
     cudaError_t e;
@@ -407,6 +403,7 @@ extern "C" int mpfc_create(const mpfc_params* p, void* d_workspace, size_t bytes
       }
     }
     if (rc == MPFC_OK) rc = mpfc_fp32_init(H);
+    if (rc == MPFC_OK) rc = mpfc_df_init(H);
   } while (0);
   if (rc != MPFC_OK) {
     mpfc_destroy(H);
@@ -512,7 +509,7 @@ static void launch_coarse(mpfc_s* H, const Lev& C, const Coef& k, cudaStream_t s
 // First level run by the tail kernel: the finest level of at most shape.tail_cells
 // cells, leaving at least one level above the coarsest and at most kMaxTail levels in
 // the tail; nlev when no tail is used.
-static int tail_first_level(const mpfc_s* H) {
+int mpfc_tail_first_level(const mpfc_s* H) {
   const int L = H->nlev;
   if (H->shape.tail_cells <= 0 || L < 2) return L;
   int lt = L - 1;
@@ -525,7 +522,7 @@ static int tail_first_level(const mpfc_s* H) {
 // Whether a V-cycle ends with k_smooth_res on the finest level (which then runs by
 // per-level launches and has post-sweeps), so that its residual test is k_resnorm_red.
 static bool vcycle_fuses_norm(const mpfc_s* H) {
-  const int L = H->nlev, lt = tail_first_level(H);
+  const int L = H->nlev, lt = mpfc_tail_first_level(H);
   const int down = lt < L ? lt : L - 1;
   return down >= 1 && H->p.nu2 >= 1;
 }
@@ -571,7 +568,7 @@ static void enqueue_vcycle(mpfc_s* H, cudaStream_t s) {
   const mpfc_params& p = H->p;
   const mpfc_launch_shape& sh = H->shape;
   const int L = H->nlev;
-  const int lt = tail_first_level(H);
+  const int lt = mpfc_tail_first_level(H);
   const int down = lt < L ? lt : L - 1;   // levels smoothed and restricted by per-level launches
   for (int l = 0; l < down; ++l) {
     MpfcRange range(mpfc_level_name(l));
@@ -638,6 +635,10 @@ static void enqueue_prologue(mpfc_s* H, cudaStream_t s, bool network = true) {
   if (p.guess == MPFC_GUESS_LEARNED && network) mpfc_enqueue_learned_guess(H, s);
   if (SCH == 2)
     for (int l = 1; l < H->nlev; ++l) {
+      if (H->df) {
+        mpfc_df_restrict_pk(H, l, s);
+        continue;
+      }
       const Lev& C = H->lev[l];
       mpfc_launch(H->shape, k_restrict_plane, grid_for(C.m, C.n, kBlk2d), kBlk2d, 0, s, (const double*)H->lev[l - 1].pk, C.pk,
                  C.m, C.n);
@@ -655,6 +656,7 @@ static void enqueue_commit(mpfc_s* H, cudaStream_t s) {
              H->guess.phikm2, (int)G, 1.0 / H->p.dt, (int)(H->p.model == MPFC_MODEL_PFC), H->ctl, H->info);
 }
 
+// The residual test of the FP64 V-cycle loop.
 template <int SCH>
 static void enqueue_resnorm(mpfc_s* H, int mode, cudaGraphConditionalHandle hnd, int set_cond, cudaStream_t s) {
   const Lev& L0 = H->lev[0];
@@ -673,6 +675,13 @@ static void enqueue_resnorm(mpfc_s* H, int mode, cudaGraphConditionalHandle hnd,
                 mode, hnd, set_cond);
 }
 
+// The residual test after the guess, which decides which V-cycle loop runs first.
+template <int SCH>
+static void enqueue_first_test(mpfc_s* H, cudaGraphConditionalHandle hnd, int set_cond, cudaStream_t s) {
+  if (H->df) mpfc_df_defect(H, SCH, 0, hnd, set_cond, s);
+  else enqueue_resnorm<SCH>(H, 0, hnd, set_cond, s);
+}
+
 // Body of the FP64 WHILE node: one V-cycle, then the residual test that sets the
 // loop condition.
 // The gated learned correction: the network adds its correction to the extrapolated
@@ -685,7 +694,7 @@ static void enqueue_learned_correction(mpfc_s* H, cudaGraphConditionalHandle hnd
   mpfc_enqueue_learned_guess(H, s);
   mpfc_launch(H->shape, k_guess_kappa, g0, kBlk2d, 0, s, L0, H->coef[SCH - 1][0]);
   mpfc_launch(H->shape, k_guess_mu<SCH>, g0, kBlk2d, 0, s, L0, H->coef[SCH - 1][0]);
-  enqueue_resnorm<SCH>(H, 0, hnd, set_cond, s);
+  enqueue_first_test<SCH>(H, hnd, set_cond, s);
 }
 
 static void learned_body(mpfc_s* H, int scheme, cudaStream_t s) {
@@ -704,8 +713,17 @@ static void fp64_body(mpfc_s* H, int scheme, cudaStream_t s) {
   }
 }
 
+// The same in correction form.
+static void df_body(mpfc_s* H, int scheme, cudaStream_t s) {
+  mpfc_df_vcycle(H, scheme, s);
+  mpfc_df_defect(H, scheme, 1, H->cur_handle, 1, s);
+}
+
 // Builds the step graph of one scheme:
 //   prologue -> resnorm(mode 0, sets cond) -> WHILE(cond){ V-cycle; resnorm(mode 1) } -> commit
+// In correction form the residual tests set two conditions, and a second loop of FP64
+// V-cycles follows the first, for values outside the correction form's range (a loop whose
+// condition is not set costs about 2 us).
 template <int SCH>
 static int build_step_graph(mpfc_s* H) {
   cudaStream_t cs = H->cap_stream;
@@ -723,8 +741,11 @@ static int build_step_graph(mpfc_s* H) {
     rc = mpfc_fp32_enqueue_step(H, SCH, cs, hnd);
   } else {
     const bool gated = guess_gated(H);
+    cudaGraphConditionalHandle hnd64 = hnd;
+    if (H->df) CKCAP(cudaGraphConditionalHandleCreate(&hnd64, graph, 0, 0), cs);
+    H->cur_handle64 = hnd64;
     enqueue_prologue<SCH>(H, cs, !gated);
-    enqueue_resnorm<SCH>(H, 0, hnd, 1, cs);
+    enqueue_first_test<SCH>(H, hnd, 1, cs);
     rc = MPFC_OK;
     if (gated) {   // IF(res0 >= gate){ network; kappa, mu; resnorm(mode 0, sets cond) }
       cudaGraphConditionalHandle hif;
@@ -732,7 +753,9 @@ static int build_step_graph(mpfc_s* H) {
       mpfc_launch(H->shape, k_guess_gate, dim3(1), dim3(32), 0, cs, (const Ctl*)H->ctl, H->guess_gate, hif);
       rc = mpfc_capture_conditional(H, cs, hif, cudaGraphCondTypeIf, &learned_body, SCH);
     }
-    if (rc == MPFC_OK) rc = mpfc_capture_while(H, cs, hnd, &fp64_body, SCH);
+    if (rc == MPFC_OK && H->df) rc = mpfc_capture_while(H, cs, hnd, &df_body, SCH);
+    H->cur_handle = hnd64;
+    if (rc == MPFC_OK) rc = mpfc_capture_while(H, cs, hnd64, &fp64_body, SCH);
     if (rc == MPFC_OK) enqueue_commit<SCH>(H, cs);
   }
   if (rc != MPFC_OK) {
@@ -819,10 +842,10 @@ static int step_stream_mode(mpfc_s* H, int scheme) {
   const bool gated = guess_gated(H);
   if (scheme == 1) {
     enqueue_prologue<1>(H, s, !gated);
-    enqueue_resnorm<1>(H, 0, 0, 0, s);
+    enqueue_first_test<1>(H, 0, 0, s);
   } else {
     enqueue_prologue<2>(H, s, !gated);
-    enqueue_resnorm<2>(H, 0, 0, 0, s);
+    enqueue_first_test<2>(H, 0, 0, s);
   }
   if (gated) {   // the gate read on the host
     Ctl c;
@@ -839,6 +862,11 @@ static int step_stream_mode(mpfc_s* H, int scheme) {
     CK(cudaStreamSynchronize(s));
     if (!host_continue(c)) break;
     MpfcRange vrange("V-cycle");
+    if (H->df && !c.range) {
+      mpfc_df_vcycle(H, scheme, s);
+      mpfc_df_defect(H, scheme, 1, 0, 0, s);
+      continue;
+    }
     if (scheme == 1) {
       enqueue_vcycle<1>(H, s);
       enqueue_resnorm<1>(H, 1, 0, 0, s);
@@ -900,12 +928,12 @@ extern "C" int mpfc_launch_counts(const mpfc_t* H, int scheme, int* per_step, in
   if (!H || (scheme != 1 && scheme != 2) || H->p.precision != MPFC_FP64 || H->p.guess == MPFC_GUESS_LEARNED)
     return MPFC_ERR_INVALID;
   const mpfc_params& p = H->p;
-  const int L = H->nlev, lt = tail_first_level(H);
+  const int L = H->nlev, lt = mpfc_tail_first_level(H);
   const int down = lt < L ? lt : L - 1;   // levels run by per-level launches
   // per level: nu1 + nu2 sweeps of two colours, restriction, tau, prolongation
   const int per_level = 2 * p.nu1 + 2 * p.nu2 + 3;
   // + the tail launch or the coarsest solve, + the residual test
-  if (per_cycle) *per_cycle = down * per_level + 2;
+  if (per_cycle) *per_cycle = H->df ? mpfc_df_launches_per_cycle(H) : down * per_level + 2;
   // step begin, source and guess, kappa, mu, [phi^k onto the coarse levels], residual test, commit
   if (per_step) *per_step = 6 + (scheme == 2 ? L - 1 : 0);
   return MPFC_OK;

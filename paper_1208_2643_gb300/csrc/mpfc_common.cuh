@@ -156,7 +156,8 @@ __device__ __forceinline__ double ldown(const double* p) {
 struct Ctl {
   double res0, res, tol;
   int cycles, max_cycles, fixed_cycles, status;   // status: 0 ok, 2 diverged
-  int skip, halt, slot, pad0;
+  int skip, halt, slot;
+  int range;                                      // a value left the correction form's range
   unsigned int counter;                           // last-block-done counter of reductions
   unsigned int pad1;
   double sums[kMaxSums];                          // results of the last reduction

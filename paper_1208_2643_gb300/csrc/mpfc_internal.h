@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "../../include/mpfc.h"
+#include "df_cells.cuh"
 #include "mpfc_common.cuh"
 
 // FP32 copy of one level for the inner V-cycles of the mixed-precision form.
@@ -85,6 +86,10 @@ struct mpfc_s {
   double* pf[mpfc::kMaxLevels];
   cudaGraphExec_t exec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
   cudaGraphConditionalHandle cur_handle = 0;   // handle of the graph being captured
+  // correction form of the FP64 V-cycle (df_cycle.cu)
+  mpfc::DLev dlev[mpfc::kMaxLevels];
+  bool df = false;                               // the handle's V-cycles run in correction form
+  cudaGraphConditionalHandle cur_handle64 = 0;   // loop of the FP64 V-cycle, for values outside the form's range
   int launch_mode = MPFC_LAUNCH_GRAPH;
   // set by mpfc_create from the precision (mpfc_default_launch_shape)
   mpfc_launch_shape shape = {1, 0, 0, 0, 8};
@@ -169,6 +174,18 @@ int mpfc_capture_conditional(mpfc_s* H, cudaStream_t cs, cudaGraphConditionalHan
                              void (*body_fn)(mpfc_s*, int, cudaStream_t), int scheme);
 void mpfc_enqueue_prologue(mpfc_s* H, int scheme, cudaStream_t s);
 void mpfc_enqueue_commit(mpfc_s* H, int scheme, cudaStream_t s);
+
+int mpfc_tail_first_level(const mpfc_s* H);
+
+// correction form of the FP64 V-cycle (df_cycle.cu)
+size_t mpfc_df_carve(mpfc_s* H, const mpfc_params* p, size_t* off, char* base, const mpfc::Lev* lev, double* const* px,
+                     double* const* pf, int nlev);
+bool mpfc_df_usable(const mpfc_s* H);
+int mpfc_df_init(mpfc_s* H);
+void mpfc_df_restrict_pk(mpfc_s* H, int l, cudaStream_t s);
+void mpfc_df_vcycle(mpfc_s* H, int scheme, cudaStream_t s);
+void mpfc_df_defect(mpfc_s* H, int scheme, int mode, cudaGraphConditionalHandle hnd, int set_cond, cudaStream_t s);
+int mpfc_df_launches_per_cycle(const mpfc_s* H);
 
 // mixed-precision form (fp32_inner.cu)
 size_t mpfc_fp32_carve(mpfc_s* H, const mpfc_params* p, size_t* off, char* base, int nlev);
