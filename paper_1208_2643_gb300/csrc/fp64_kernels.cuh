@@ -912,9 +912,10 @@ __global__ void k_commit(const double* __restrict__ phinew, double* phik, double
 }
 
 // ---------------------------------------------------------------------------
-// Diagnostics: mass and energy sums, Poisson multigrid for the -1 norm.
+// Diagnostics: mass and energy sums.
 // ---------------------------------------------------------------------------
 static __global__ void k_sum1(const double* __restrict__ f, int G, Ctl* ctl, double* partials) {
+  pdl_enter();
   double v[1] = {0.0};
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < G; t += gridDim.x * blockDim.x) v[0] += f[t];
   if (grid_sum<1>(v, partials, &ctl->counter)) ctl->sums[0] = v[0];
@@ -954,110 +955,6 @@ static __global__ void k_energy_sums(const double* __restrict__ phi, const doubl
   }
   if (grid_sum<7>(v, partials, &ctl->counter))
     for (int s = 0; s < 7; ++s) ctl->sums[s] = v[s];
-}
-
-// x = f - mean: the right-hand side of the mean-zero Poisson problem
-static __global__ void k_sub_mean(const double* __restrict__ f, double* __restrict__ out, int G, const Ctl* ctl) {
-  double mean = ctl->sums[0] / (double)G;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < G; t += gridDim.x * blockDim.x) out[t] = f[t] - mean;
-}
-
-// Red-black Gauss-Seidel half sweep for -Delta_h x = f (periodic, or Neumann in y:
-// a boundary row's ghost is its own unknown, so it has three neighbours).
-static __global__ void k_pois_smooth(double* __restrict__ x, const double* __restrict__ f, int m, int n, int nyn,
-                                     double h2, int color) {
-  int xi = blockIdx.x * blockDim.x + threadIdx.x;
-  int j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (xi >= (m >> 1) || j >= n) return;
-  int i = 2 * xi + ((j + color) & 1);
-  int im = wrapm(i - 1, m), ip = wrapm(i + 1, m), jm = ywrap(j - 1, n, nyn), jp = ywrap(j + 1, n, nyn);
-  double s = (x[j * m + im] + x[j * m + ip]) + (x[jm * m + i] + x[jp * m + i]);
-  if (nyn && (j == 0 || j == n - 1)) {
-    s -= x[j * m + i];
-    x[j * m + i] = (s + h2 * f[j * m + i]) / 3.0;
-  } else {
-    x[j * m + i] = 0.25 * (s + h2 * f[j * m + i]);
-  }
-}
-
-// coarse f = R (f + Delta_h x), coarse x = 0; also the sum of squared fine residuals
-static __global__ void k_pois_restrict(const double* __restrict__ x, const double* __restrict__ f, double* __restrict__ fc,
-                                double* __restrict__ xc, int mc, int nc, int nyn, double ih2) {
-  int I = blockIdx.x * blockDim.x + threadIdx.x;
-  int J = blockIdx.y * blockDim.y + threadIdx.y;
-  if (I >= mc || J >= nc) return;
-  int m = 2 * mc, n = 2 * nc;
-  double acc = 0.0;
-  for (int dj = 0; dj < 2; ++dj)
-    for (int di = 0; di < 2; ++di) {
-      int i = 2 * I + di, j = 2 * J + dj;
-      int im = wrapm(i - 1, m), ip = wrapm(i + 1, m), jm = ywrap(j - 1, n, nyn), jp = ywrap(j + 1, n, nyn);
-      double lap = ((x[j * m + im] + x[j * m + ip]) + (x[jm * m + i] + x[jp * m + i]) - 4.0 * x[j * m + i]) * ih2;
-      acc += f[j * m + i] + lap;
-    }
-  fc[J * mc + I] = 0.25 * acc;
-  xc[J * mc + I] = 0.0;
-}
-
-static __global__ void k_pois_prolong(const double* __restrict__ xc, double* __restrict__ x, int mc, int nc, int nyn) {
-  int I = blockIdx.x * blockDim.x + threadIdx.x;
-  int J = blockIdx.y * blockDim.y + threadIdx.y;
-  if (I >= mc || J >= nc) return;
-  int Im = wrapm(I - 1, mc), Ip = wrapm(I + 1, mc), Jm = ywrap(J - 1, nc, nyn), Jp = ywrap(J + 1, nc, nyn);
-  auto X = [&](int a, int b) { return xc[b * mc + a]; };
-  double e00 = X(I, J), eW = X(Im, J), eE = X(Ip, J), eS = X(I, Jm), eN = X(I, Jp);
-  double eSW = X(Im, Jm), eSE = X(Ip, Jm), eNW = X(Im, Jp), eNE = X(Ip, Jp);
-  const double w9 = 9.0 / 16.0, w3 = 3.0 / 16.0, w1 = 1.0 / 16.0;
-  int mf = 2 * mc;
-  size_t f00 = (size_t)(2 * J) * mf + 2 * I, f01 = f00 + mf;
-  x[f00] += fma(w9, e00, fma(w3, eW + eS, w1 * eSW));
-  x[f00 + 1] += fma(w9, e00, fma(w3, eE + eS, w1 * eSE));
-  x[f01] += fma(w9, e00, fma(w3, eW + eN, w1 * eNW));
-  x[f01 + 1] += fma(w9, e00, fma(w3, eE + eN, w1 * eNE));
-}
-
-// Coarsest Poisson level: `sweeps` red-black sweeps in one CTA, then the mean removed.
-static __global__ void k_pois_coarse(double* x, const double* f, int m, int n, int nyn, double h2, int sweeps) {
-  extern __shared__ double xs[];
-  int G = m * n;
-  for (int t = threadIdx.x; t < G; t += blockDim.x) xs[t] = x[t];
-  __syncthreads();
-  for (int s = 0; s < sweeps; ++s)
-    for (int color = 0; color < 2; ++color) {
-      for (int t = threadIdx.x; t < G; t += blockDim.x) {
-        int i = t % m, j = t / m;
-        if (((i + j) & 1) != color) continue;
-        if (nyn && (j == 0 || j == n - 1)) xs[t] = (nbsum_s(xs, m, n, t, nyn) - xs[t] + h2 * f[t]) / 3.0;
-        else xs[t] = 0.25 * (nbsum_s(xs, m, n, t, nyn) + h2 * f[t]);
-      }
-      __syncthreads();
-    }
-  if (threadIdx.x == 0) {
-    double mean = 0.0;
-    for (int t = 0; t < G; ++t) mean += xs[t];
-    xs[G] = mean / G;
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < G; t += blockDim.x) x[t] = xs[t] - xs[G];
-}
-
-// sum of squared residuals of -Delta_h x = f, and sum of f^2
-static __global__ void k_pois_resnorm(const double* __restrict__ x, const double* __restrict__ f, int m, int n, int nyn,
-                               double ih2, Ctl* ctl, double* partials) {
-  double v[2] = {0.0, 0.0};
-  int G = m * n;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < G; t += gridDim.x * blockDim.x) {
-    int i = t % m, j = t / m;
-    int im = wrapm(i - 1, m), ip = wrapm(i + 1, m), jm = ywrap(j - 1, n, nyn), jp = ywrap(j + 1, n, nyn);
-    double lap = ((x[j * m + im] + x[j * m + ip]) + (x[jm * m + i] + x[jp * m + i]) - 4.0 * x[t]) * ih2;
-    double r = f[t] + lap;
-    v[0] += r * r;
-    v[1] += f[t] * f[t];
-  }
-  if (grid_sum<2>(v, partials, &ctl->counter)) {
-    ctl->sums[0] = v[0];
-    ctl->sums[1] = v[1];
-  }
 }
 
 #include "fp64_tail.cuh"

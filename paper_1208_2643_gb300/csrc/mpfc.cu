@@ -243,6 +243,7 @@ static size_t carve(mpfc_s* H, const mpfc_params* p, char* base) {
   int Gc = lev[L - 1].m * lev[L - 1].n;
   float* K3a = c.take<float>(2 * (size_t)Gc * Gc);   // K3 and c L of scheme 1 (mpfc_coarse_block)
   float* K3b = c.take<float>(2 * (size_t)Gc * Gc);
+  float* poisP = c.take<float>((size_t)Gc * Gc);
   mpfc_fp32_carve(H, p, &c.off, base, L);
   mpfc_df_carve(H, p, &c.off, base, lev, px, pf, L);
   mpfc_guess_carve(H, p, &c.off, base);
@@ -266,6 +267,7 @@ static size_t carve(mpfc_s* H, const mpfc_params* p, char* base) {
     H->pin_active = 0;
     H->K3[0] = K3a;
     H->K3[1] = K3b;
+    H->poisP = poisP;
   }
   return c.off;
 }
@@ -404,6 +406,7 @@ extern "C" int mpfc_create(const mpfc_params* p, void* d_workspace, size_t bytes
     }
     if (rc == MPFC_OK) rc = mpfc_fp32_init(H);
     if (rc == MPFC_OK) rc = mpfc_df_init(H);
+    if (rc == MPFC_OK) rc = mpfc_pois_init(H);
   } while (0);
   if (rc != MPFC_OK) {
     mpfc_destroy(H);
@@ -425,6 +428,7 @@ void mpfc_drop_graphs(mpfc_s* H) {
 extern "C" void mpfc_destroy(mpfc_t* H) {
   if (!H) return;
   mpfc_drop_graphs(H);
+  if (H->pois_exec) cudaGraphExecDestroy(H->pois_exec);
   mpfc_fp32_destroy(H);
   if (H->cap_stream) cudaStreamDestroy(H->cap_stream);
   if (H->body_stream) cudaStreamDestroy(H->body_stream);
@@ -1092,53 +1096,14 @@ extern "C" int mpfc_mass(mpfc_t* H, double* out) {
   return MPFC_OK;
 }
 
-// Periodic Poisson multigrid: -Delta_h x = f (f mean-zero), V(2,2) red-black
-// cycles until ||r|| <= 1e-13 ||f|| (at most 60).  Result in H->px[0].
-static int poisson_solve(mpfc_s* H, const double* rhs) {
-  int L = H->nlev;
-  size_t G0 = (size_t)H->p.m * H->p.n;
-  cudaStream_t s = H->stream;
-  k_sum1<<<mpfc_reduce_blocks(G0), 256, 0, s>>>(rhs, (int)G0, H->ctl, H->partials);
-  k_sub_mean<<<mpfc_reduce_blocks(G0), 256, 0, s>>>(rhs, H->pf[0], (int)G0, H->ctl);
-  CK(cudaMemsetAsync(H->px[0], 0, G0 * sizeof(double), s));
-  for (int cyc = 0; cyc < 60; ++cyc) {
-    for (int l = 0; l < L - 1; ++l) {
-      const Lev& F = H->lev[l];
-      dim3 g = grid_for(F.m / 2, F.n, kBlk2d);
-      for (int sw = 0; sw < 2; ++sw)
-        for (int c = 0; c < 2; ++c) k_pois_smooth<<<g, kBlk2d, 0, s>>>(H->px[l], H->pf[l], F.m, F.n, F.nyn, F.h * F.h, c);
-      const Lev& C = H->lev[l + 1];
-      k_pois_restrict<<<grid_for(C.m, C.n, kBlk2d), kBlk2d, 0, s>>>(H->px[l], H->pf[l], H->pf[l + 1], H->px[l + 1],
-                                                                     C.m, C.n, C.nyn, 1.0 / (F.h * F.h));
-    }
-    const Lev& Cc = H->lev[L - 1];
-    k_pois_coarse<<<1, 128, sizeof(double) * (Cc.m * Cc.n + 1), s>>>(H->px[L - 1], H->pf[L - 1], Cc.m, Cc.n,
-                                                                      Cc.nyn, Cc.h * Cc.h, 200);
-    for (int l = L - 2; l >= 0; --l) {
-      const Lev& F = H->lev[l];
-      const Lev& C = H->lev[l + 1];
-      k_pois_prolong<<<grid_for(C.m, C.n, kBlk2d), kBlk2d, 0, s>>>(H->px[l + 1], H->px[l], C.m, C.n, C.nyn);
-      dim3 g = grid_for(F.m / 2, F.n, kBlk2d);
-      for (int sw = 0; sw < 2; ++sw)
-        for (int c = 0; c < 2; ++c) k_pois_smooth<<<g, kBlk2d, 0, s>>>(H->px[l], H->pf[l], F.m, F.n, F.nyn, F.h * F.h, c);
-    }
-    const Lev& F0 = H->lev[0];
-    k_pois_resnorm<<<mpfc_reduce_blocks(G0), 256, 0, s>>>(H->px[0], H->pf[0], F0.m, F0.n, F0.nyn,
-                                                          1.0 / (F0.h * F0.h), H->ctl, H->partials);
-    CK(cudaGetLastError());
-    double v[2];
-    int rc = read_sums(H, v, 2);
-    if (rc) return rc;
-    if (!(v[0] == v[0])) return MPFC_ERR_DIVERGED;
-    if (v[0] <= 1e-26 * v[1] || v[1] == 0.0) break;
-  }
-  return MPFC_OK;
-}
-
 extern "C" int mpfc_energy(mpfc_t* H, mpfc_energy_t* out) {
   if (!H || !out) return MPFC_ERR_INVALID;
-  int rc = poisson_solve(H, H->psik);
+  int rc = mpfc_pois_solve(H);
   if (rc) return rc;
+  double q[1];   // squared residual of the Poisson solve
+  rc = read_sums(H, q, 1);
+  if (rc) return rc;
+  if (!(q[0] == q[0])) return MPFC_ERR_DIVERGED;
   size_t G = (size_t)H->p.m * H->p.n;
   k_energy_sums<<<mpfc_reduce_blocks(G), 256, 0, H->stream>>>(
       H->phik, H->phikm1, H->psik, H->px[0], H->p.m, H->p.n, H->lev[0].nyn, H->pin_active ? H->pinW[0] : nullptr,

@@ -93,6 +93,10 @@ struct mpfc_s {
   int launch_mode = MPFC_LAUNCH_GRAPH;
   // set by mpfc_create from the precision (mpfc_default_launch_shape)
   mpfc_launch_shape shape = {1, 0, 0, 0, 8};
+  // Poisson solve of the energies (poisson.cu)
+  float* poisP = nullptr;               // coarsest grid's pseudo-inverse (FP32, G x G)
+  cudaGraphExec_t pois_exec = nullptr;
+  mpfc_launch_shape pshape = {4, 0, 0, 0, 1, 0};
   // mixed precision
   Lev32 lev32[mpfc::kMaxLevels];
   float* K3f[2] = {nullptr, nullptr};
@@ -186,6 +190,10 @@ void mpfc_df_restrict_pk(mpfc_s* H, int l, cudaStream_t s);
 void mpfc_df_vcycle(mpfc_s* H, int scheme, cudaStream_t s);
 void mpfc_df_defect(mpfc_s* H, int scheme, int mode, cudaGraphConditionalHandle hnd, int set_cond, cudaStream_t s);
 int mpfc_df_launches_per_cycle(const mpfc_s* H);
+
+// Poisson solve of the -1 norm (poisson.cu)
+int mpfc_pois_init(mpfc_s* H);
+int mpfc_pois_solve(mpfc_s* H);
 
 // mixed-precision form (fp32_inner.cu)
 size_t mpfc_fp32_carve(mpfc_s* H, const mpfc_params* p, size_t* off, char* base, int nlev);
