@@ -12,6 +12,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "df_kernels.cuh"
 #include "fp64_kernels.cuh"
 #include "mpfc_internal.h"
 
@@ -26,7 +27,8 @@ struct BItem {
 struct BCtl {                // per instance
   double res0, res;
   int cycles, status, active, halted;
-  int total_cycles, steps, first_error, pad;
+  int total_cycles, steps, first_error;
+  int range;                 // a value left the correction form's range: FP64 V-cycles
 };
 
 struct BGlobal {
@@ -172,8 +174,28 @@ __global__ void kb_step_begin(BCtl* ctl, int count) {
   if (i < count) {
     ctl[i].cycles = 0;
     ctl[i].status = 0;
+    ctl[i].range = 0;
     ctl[i].active = !ctl[i].halted;
   }
+}
+
+// Takes in an instance's residual norm.
+__device__ __forceinline__ void inst_residual(BCtl& c, double res, int mode, const BGlobal* glob) {
+  if (mode == 0) {
+    if (!c.halted) {
+      c.res0 = res;
+      c.res = res;
+      if (!(res == res) || isinf(res)) c.status = 2;
+    }
+  } else if (c.active) {
+    c.res = res;
+    c.cycles += 1;
+    if (!(res == res) || isinf(res) || res > 1e10 * fmax(c.res0, glob->tol)) c.status = 2;
+  }
+}
+__device__ __forceinline__ bool inst_continues(const BCtl& c, const BGlobal* glob) {
+  return !c.halted && c.status == 0 &&
+         (glob->fixed_cycles > 0 ? c.cycles < glob->fixed_cycles : (c.res > glob->tol && c.cycles < glob->max_cycles));
 }
 
 // Per-instance scaled residual norms.  mode 0: after the guess; mode 1: after a
@@ -220,23 +242,9 @@ __global__ void __launch_bounds__(256) kb_resnorm(const BItem* __restrict__ item
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if (lane == 0) {
       BCtl& c = ctl[inst];
-      Lev L = levs[inst * kMaxLevels];
-      double res = sqrt(s / (3.0 * (double)L.m * (double)L.n));
-      if (mode == 0) {
-        if (!c.halted) {
-          c.res0 = res;
-          c.res = res;
-          if (!(res == res) || isinf(res)) c.status = 2;
-        }
-      } else if (c.active) {
-        c.res = res;
-        c.cycles += 1;
-        if (!(res == res) || isinf(res) || res > 1e10 * fmax(c.res0, glob->tol)) c.status = 2;
-      }
-      bool act = !c.halted && c.status == 0 &&
-                 (glob->fixed_cycles > 0 ? c.cycles < glob->fixed_cycles
-                                         : (c.res > glob->tol && c.cycles < glob->max_cycles));
-      c.active = act ? 1 : 0;
+      const Lev& L = levs[inst * kMaxLevels];
+      inst_residual(c, sqrt(s / (3.0 * (double)L.m * (double)L.n)), mode, glob);
+      c.active = inst_continues(c, glob) ? 1 : 0;
     }
   }
   __syncthreads();
@@ -247,6 +255,190 @@ __global__ void __launch_bounds__(256) kb_resnorm(const BItem* __restrict__ item
     glob->counter = 0u;
     if (set_cond) cudaGraphSetConditional(hnd, any ? 1u : 0u);
   }
+}
+
+// ---------------------------------------------------------------------------
+// The V-cycle in correction form (df_cells.cuh) over the same work lists.
+// ---------------------------------------------------------------------------
+// FINAL: the last post-sweep; on an instance's finest level it adds the correction to u.
+// A block of at most kHalfThreads threads strides over its tx x ty tile.
+constexpr int kHalfThreads = 512;
+template <int SCH, int MODE, bool FINAL>
+__global__ void __launch_bounds__(kHalfThreads) kb_df_half(const BItem* __restrict__ items, int n,
+                                                           const DPar* __restrict__ pars, const Lev* __restrict__ levs,
+                                                           const BCtl* __restrict__ ctl, int color, int tx, int ty) {
+  for (int it = blockIdx.x; it < n; it += gridDim.x) {
+    const BItem w = items[it];
+    if (!ctl[w.inst].active) continue;
+    const int id = w.inst * kMaxLevels + w.level;
+    const DPar& P = pars[id];
+    const int x1 = min(w.x0 + tx, P.L.m >> 1), y1 = min(w.y0 + ty, P.L.n);
+    for (int j = w.y0 + threadIdx.y; j < y1; j += blockDim.y)
+      for (int x = w.x0 + threadIdx.x; x < x1; x += blockDim.x) {
+        if (FINAL && w.level == 0) {
+          double* const u[3] = {levs[id].phi, levs[id].mu, levs[id].ka};
+          df_smooth_cell<SCH, MODE, false, true>(P, color, x, j, u);
+        } else {
+          df_smooth_cell<SCH, MODE, false, false>(P, color, x, j);
+        }
+      }
+  }
+}
+dim3 half_block(int tx, int ty) {
+  const int bx = std::min(tx, kHalfThreads);
+  return dim3(bx, std::max(1, std::min(ty, kHalfThreads / bx)));
+}
+
+template <int SCH>
+__global__ void __launch_bounds__(kPTX * kPTY) kb_df_restrict(const BItem* __restrict__ items, int n,
+                                                              const DPar* __restrict__ pars,
+                                                              const BCtl* __restrict__ ctl, int zero) {
+  for (int it = blockIdx.x; it < n; it += gridDim.x) {
+    const BItem w = items[it];
+    if (!ctl[w.inst].active) continue;
+    const int idc = w.inst * kMaxLevels + w.level;
+    const DPar& C = pars[idc];
+    const int I = w.x0 + threadIdx.x, J = w.y0 + threadIdx.y;
+    if (I < C.L.m && J < C.L.n) df_restrict_cell<SCH, true, true>(pars[idc - 1], C, I, J, zero);
+  }
+}
+
+__global__ void __launch_bounds__(kPTX * kPTY) kb_df_prolong(const BItem* __restrict__ items, int n,
+                                                             const DPar* __restrict__ pars, const BCtl* __restrict__ ctl) {
+  for (int it = blockIdx.x; it < n; it += gridDim.x) {
+    const BItem w = items[it];
+    if (!ctl[w.inst].active) continue;
+    const int idc = w.inst * kMaxLevels + w.level;
+    const DPar& C = pars[idc];
+    const int I = w.x0 + threadIdx.x, J = w.y0 + threadIdx.y;
+    if (I >= C.L.m || J >= C.L.n) continue;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) df_prolong_plane(C.L, pars[idc - 1].L, c, I, J);
+  }
+}
+
+// phi^k of a coarse level in float-float, from the FP64 plane that kb_restrict_pk wrote.
+__global__ void kb_df_pk(const BItem* __restrict__ items, int n, const DPar* __restrict__ pars, const Lev* __restrict__ levs,
+                         const BCtl* __restrict__ ctl) {
+  for (int it = blockIdx.x; it < n; it += gridDim.x) {
+    const BItem w = items[it];
+    if (ctl[w.inst].halted) continue;
+    const int id = w.inst * kMaxLevels + w.level;
+    const DLev& C = pars[id].L;
+    const int I = w.x0 + threadIdx.x, J = w.y0 + threadIdx.y;
+    if (I < C.m && J < C.n) C.pk[dindex(C, I, J)] = f2(df_of(levs[id].pk[(size_t)J * C.m + I]));
+  }
+}
+
+// The last `tail` levels of each instance in one CTA (tail >= 2), or its coarsest solve alone.
+template <int SCH>
+__global__ void __launch_bounds__(kDfTailThreads, 1) kb_df_tail(const DPar* __restrict__ pars, const int* __restrict__ nlev,
+                                                                const float* __restrict__ K3,
+                                                                const long long* __restrict__ K3off,
+                                                                const BCtl* __restrict__ ctl, int tail, int nu1, int nu2) {
+  extern __shared__ float2 tsm[];
+  __shared__ DPar sl[kDfTailMax];
+  const int inst = blockIdx.x;
+  if (!ctl[inst].active) return;
+  const DPar* lv = pars + inst * kMaxLevels + nlev[inst] - tail;
+  df_tail_body<SCH, false>(DTailDim{tail, nu1, nu2, 0}, lv, K3 + K3off[inst], tsm, sl, [] {});
+}
+template <int SCH>
+__global__ void __launch_bounds__(32) kb_df_coarse(const DPar* __restrict__ pars, const int* __restrict__ nlev,
+                                                   const float* __restrict__ K3, const long long* __restrict__ K3off,
+                                                   const BCtl* __restrict__ ctl) {
+  extern __shared__ float2 tsm[];
+  const int inst = blockIdx.x;
+  if (!ctl[inst].active) return;
+  coarse_df_warp<SCH>(pars[inst * kMaxLevels + nlev[inst] - 1], K3 + K3off[inst], tsm);
+}
+
+// u += d of the instances whose finest level took no final half sweep (it is in the tail, or
+// `all`).
+__global__ void kb_df_apply(const BItem* __restrict__ items, int n, const DPar* __restrict__ pars,
+                            const Lev* __restrict__ levs, const int* __restrict__ nlev, const BCtl* __restrict__ ctl,
+                            int tail, int all) {
+  for (int it = blockIdx.x; it < n; it += gridDim.x) {
+    const BItem w = items[it];
+    if (!ctl[w.inst].active || (!all && nlev[w.inst] > tail)) continue;
+    const int id = w.inst * kMaxLevels;
+    const DLev& D = pars[id].L;
+    const Lev& L = levs[id];
+    const int i = w.x0 + threadIdx.x, j = w.y0 + threadIdx.y;
+    if (i >= D.m || j >= D.n) continue;
+    const size_t q = dindex(D, i, j), t = (size_t)j * D.m + i;
+    L.phi[t] += df_to_f64(ldd(D.d[0] + q));
+    L.mu[t] += df_to_f64(ldd(D.d[1] + q));
+    L.ka[t] += df_to_f64(ldd(D.d[2] + q));
+  }
+}
+
+// kb_resnorm with the correction form's inputs (df_defect_cell).  An instance with a value
+// outside the form's range stops here and continues in the FP64 loop (kb_take64).
+template <int SCH, bool MODE0>
+__global__ void __launch_bounds__(256) kb_df_defect(const BItem* __restrict__ items, int n, const int* __restrict__ ibeg,
+                                                    int count, const Lev* __restrict__ levs,
+                                                    const Coef* __restrict__ coefs, const DPar* __restrict__ pars, BCtl* ctl,
+                                                    BGlobal* glob, double* partials, int zero,
+                                                    cudaGraphConditionalHandle hnd, cudaGraphConditionalHandle hnd64) {
+  __shared__ double red[32];
+  __shared__ bool last;
+  for (int it = blockIdx.x; it < n; it += gridDim.x) {
+    const BItem w = items[it];
+    double v = 0.0;
+    if (MODE0 ? !ctl[w.inst].halted : (bool)ctl[w.inst].active) {
+      const int id = w.inst * kMaxLevels;
+      const Lev& L = levs[id];
+      const int i = w.x0 + threadIdx.x, j = w.y0 + threadIdx.y;
+      if (i < L.m && j < L.n) {
+        bool bad = false;
+        v = df_defect_cell<SCH, MODE0, true>(L, coefs[id], pars[id], i, j, zero, bad);
+        if (bad) atomicOr(&ctl[w.inst].range, 1);
+      }
+    }
+    const double tot = block_total2d(v, red);
+    if (threadIdx.x == 0 && threadIdx.y == 0) partials[it] = tot;
+  }
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    __threadfence();
+    last = (atomicAdd(&glob->counter, 1u) == gridDim.x - 1);
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const int lane = tid & 31, wid = tid >> 5, nw = (blockDim.x * blockDim.y) >> 5;
+  for (int inst = wid; inst < count; inst += nw) {
+    double s = 0.0;
+    for (int it = ibeg[inst] + lane; it < ibeg[inst + 1]; it += 32) s += ((volatile double*)partials)[it];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+      BCtl& c = ctl[inst];
+      const Lev& L = levs[inst * kMaxLevels];
+      const int range = *(volatile int*)&c.range;
+      inst_residual(c, sqrt(s / (3.0 * (double)L.m * (double)L.n)), MODE0 ? 0 : 1, glob);
+      const bool go = inst_continues(c, glob);
+      c.range = range | (go && c.res < kDfMinResidual);
+      c.active = go && !c.range;
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    int any = 0, any64 = 0;
+    for (int inst = 0; inst < count; ++inst) {
+      any |= ctl[inst].active;
+      any64 |= ctl[inst].range && inst_continues(ctl[inst], glob);
+    }
+    glob->counter = 0u;
+    cudaGraphSetConditional(hnd, any ? 1u : 0u);
+    cudaGraphSetConditional(hnd64, any64 ? 1u : 0u);
+  }
+}
+
+// Start of an FP64 V-cycle: the instances that left the correction form are active.
+__global__ void kb_take64(BCtl* ctl, const BGlobal* glob, int count) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < count) ctl[i].active = inst_continues(ctl[i], glob);
 }
 
 // psi update and history rotation per instance (level-0 items); a failing instance
@@ -327,6 +519,12 @@ struct mpfc_batch_s {
   Lev* d_lev = nullptr;
   Coef* d_coef[2] = {nullptr, nullptr};
   SourceArgs* d_src[2] = {nullptr, nullptr};
+  // correction form: every instance has at least two levels and coefficients in its range
+  bool df = false;
+  int tail = 1;                    // levels of each instance in the coarse tail (1: the coarsest solve alone)
+  size_t tail_smem = 0;
+  DPar* d_par[2] = {nullptr, nullptr};
+  std::vector<DLev> dlev;          // [inst * kMaxLevels + l]
   int* d_nlev = nullptr;
   float* d_K3[2] = {nullptr, nullptr};
   long long* d_K3off = nullptr;
@@ -469,6 +667,8 @@ size_t carve_batch(mpfc_batch_s* B, int count, const mpfc_params* each, char* ba
   Coef* d_c2 = c.take<Coef>((size_t)count * kMaxLevels);
   SourceArgs* d_s1 = c.take<SourceArgs>(count);
   SourceArgs* d_s2 = c.take<SourceArgs>(count);
+  DPar* d_p1 = c.take<DPar>((size_t)count * kMaxLevels);
+  DPar* d_p2 = c.take<DPar>((size_t)count * kMaxLevels);
   int* d_nlev = c.take<int>(count);
   long long* d_K3off = c.take<long long>(count);
   double* d_inv_s = c.take<double>(count);
@@ -493,6 +693,9 @@ size_t carve_batch(mpfc_batch_s* B, int count, const mpfc_params* each, char* ba
     B->d_coef[1] = d_c2;
     B->d_src[0] = d_s1;
     B->d_src[1] = d_s2;
+    B->d_par[0] = d_p1;
+    B->d_par[1] = d_p2;
+    B->dlev.assign((size_t)count * kMaxLevels, DLev{});
     B->d_nlev = d_nlev;
     B->d_K3off = d_K3off;
     B->d_inv_s = d_inv_s;
@@ -542,7 +745,30 @@ size_t carve_batch(mpfc_batch_s* B, int count, const mpfc_params* each, char* ba
         v.b1 = v.b2 = v.b3 = nullptr;
         v.pk = phik;
       }
-      if (B && base) B->lev[(size_t)i * kMaxLevels + l] = v;
+      // planes of the correction form: the finest level's own, the coarser levels' in the FP64
+      // V-cycle's planes, which it writes before it reads them
+      DLev d;
+      memset(&d, 0, sizeof(d));
+      d.m = m;
+      d.n = n;
+      if (l > 0) {
+        double* const planes[8] = {v.phi, v.mu, v.ka, v.S1, v.S2, v.S3, v.b1, v.b2};
+        for (int q = 0; q < 3; ++q) {
+          d.d[q] = reinterpret_cast<float2*>(planes[q]);
+          d.r[q] = reinterpret_cast<float2*>(planes[3 + q]);
+        }
+        d.pb = reinterpret_cast<float2*>(planes[6]);
+        d.pk = reinterpret_cast<float2*>(planes[7]);
+      } else if (nl[i] > 1) {
+        for (int q = 0; q < 3; ++q) d.d[q] = c.take<float2>(G);
+        for (int q = 0; q < 3; ++q) d.r[q] = c.take<float2>(G);
+        d.pb = c.take<float2>(G);
+        d.pk = c.take<float2>(G);
+      }
+      if (B && base) {
+        B->lev[(size_t)i * kMaxLevels + l] = v;
+        B->dlev[(size_t)i * kMaxLevels + l] = d;
+      }
       m /= 2;
       n /= 2;
       h *= 2.0;
@@ -594,6 +820,59 @@ void enqueue_batch_vcycle(mpfc_batch_s* B, cudaStream_t s) {
   }
 }
 
+// The same in correction form; each restriction and each residual also runs the first red half
+// sweep of the level it feeds.
+template <int SCH>
+void enqueue_batch_df_vcycle(mpfc_batch_s* B, cudaStream_t s) {
+  const int S = SCH - 1;
+  const mpfc_params& p = B->p0;
+  const DPar* pars = B->d_par[S];
+  const int gt = B->GL - B->tail;   // first global level of the tail
+  auto half = [&](auto kern, int gl, int color) {
+    const int n = B->half_cnt[gl];
+    if (n)
+      kern<<<grid_for_items(n), half_block(B->tile_x[gl], B->tile_y[gl]), 0, s>>>(
+          B->d_items + B->half_off[gl], n, pars, B->d_lev, B->d_ctl, color, B->tile_x[gl], B->tile_y[gl]);
+  };
+  const dim3 blk2(kPTX, kPTY);
+  for (int gl = 0; gl < gt; ++gl) {
+    if (p.nu1 > 0) {
+      half(kb_df_half<SCH, kOwn, false>, gl, 1);
+      for (int sw = 1; sw < p.nu1; ++sw)
+        for (int color = 0; color < 2; ++color) half(kb_df_half<SCH, kGen, false>, gl, color);
+    }
+    const int n = B->full_cnt[gl + 1];
+    if (n)
+      kb_df_restrict<SCH><<<grid_for_items(n), blk2, 0, s>>>(B->d_items + B->full_off[gl + 1], n, pars, B->d_ctl,
+                                                             p.nu1 == 0);
+  }
+  if (B->tail >= 2)
+    kb_df_tail<SCH><<<B->count, kDfTailThreads, B->tail_smem, s>>>(pars, B->d_nlev, B->d_K3[S], B->d_K3off, B->d_ctl,
+                                                                 B->tail, p.nu1, p.nu2);
+  else
+    kb_df_coarse<SCH><<<B->count, 32, B->tail_smem, s>>>(pars, B->d_nlev, B->d_K3[S], B->d_K3off, B->d_ctl);
+  for (int gl = gt - 1; gl >= 0; --gl) {
+    const int n = B->full_cnt[gl + 1];
+    if (n) kb_df_prolong<<<grid_for_items(n), blk2, 0, s>>>(B->d_items + B->full_off[gl + 1], n, pars, B->d_ctl);
+    for (int sw = 0; sw < p.nu2; ++sw)
+      for (int color = 0; color < 2; ++color) {
+        if (sw == p.nu2 - 1) half(kb_df_half<SCH, kGen, true>, gl, color);
+        else half(kb_df_half<SCH, kGen, false>, gl, color);
+      }
+  }
+  if (p.nu2 == 0 || *std::min_element(B->nlev.begin(), B->nlev.end()) <= B->tail)
+    kb_df_apply<<<grid_for_items(B->fin_cnt), blk2, 0, s>>>(B->d_items + B->fin_off, B->fin_cnt, pars, B->d_lev, B->d_nlev,
+                                                            B->d_ctl, B->tail, p.nu2 == 0);
+}
+
+template <int SCH, bool MODE0>
+void enqueue_batch_df_defect(mpfc_batch_s* B, cudaGraphConditionalHandle hnd, cudaGraphConditionalHandle hnd64,
+                             cudaStream_t s) {
+  kb_df_defect<SCH, MODE0><<<grid_for_items(B->fin_cnt), dim3(kPTX, kPTY), 0, s>>>(
+      B->d_items + B->fin_off, B->fin_cnt, B->d_ibeg, B->count, B->d_lev, B->d_coef[SCH - 1], B->d_par[SCH - 1], B->d_ctl,
+      B->d_glob, B->d_partials, B->p0.nu1 == 0, hnd, hnd64);
+}
+
 template <int SCH>
 void enqueue_batch_resnorm(mpfc_batch_s* B, int mode, cudaGraphConditionalHandle hnd, int set_cond, cudaStream_t s) {
   kb_resnorm<SCH><<<grid_for_items(B->fin_cnt), dim3(kPTX, kPTY), 0, s>>>(
@@ -614,6 +893,8 @@ void enqueue_batch_prologue(mpfc_batch_s* B, cudaStream_t s) {
       int n = B->full_cnt[gl];
       if (n)
         kb_restrict_pk<<<grid_for_items(n), blk2, 0, s>>>(B->d_items + B->full_off[gl], n, B->d_lev, B->d_ctl);
+      if (n && B->df)
+        kb_df_pk<<<grid_for_items(n), blk2, 0, s>>>(B->d_items + B->full_off[gl], n, B->d_par[1], B->d_lev, B->d_ctl);
     }
   kb_guess<SCH><<<g, blk2, 0, s>>>(fin, B->fin_cnt, B->d_lev, B->d_coef[SCH - 1], B->d_ctl, 0);
   kb_guess<SCH><<<g, blk2, 0, s>>>(fin, B->fin_cnt, B->d_lev, B->d_coef[SCH - 1], B->d_ctl, 1);
@@ -627,6 +908,31 @@ void enqueue_batch_commit(mpfc_batch_s* B, cudaStream_t s) {
   kb_step_end<<<(B->count + 127) / 128, 128, 0, s>>>(B->d_ctl, B->d_glob, B->count);
 }
 
+// A WHILE node on condition hnd after what the capture on B->cap holds so far; body(stream)
+// enqueues its kernels.
+template <typename Body>
+int capture_loop(mpfc_batch_s* B, cudaGraphConditionalHandle hnd, Body body_fn) {
+  cudaStream_t cs = B->cap;
+  cudaGraph_t graph = nullptr;
+  cudaStreamCaptureStatus st;
+  const cudaGraphNode_t* deps = nullptr;
+  size_t ndeps = 0;
+  BCK(cudaStreamGetCaptureInfo(cs, &st, nullptr, &graph, &deps, nullptr, &ndeps));
+  std::vector<cudaGraphNode_t> dv(deps, deps + ndeps);
+  cudaGraphNodeParams cp = {cudaGraphNodeTypeConditional};
+  cp.conditional.handle = hnd;
+  cp.conditional.type = cudaGraphCondTypeWhile;
+  cp.conditional.size = 1;
+  cudaGraphNode_t cnode;
+  BCK(cudaGraphAddNode(&cnode, graph, dv.data(), nullptr, dv.size(), &cp));
+  cudaGraph_t body = cp.conditional.phGraph_out[0];
+  BCK(cudaStreamUpdateCaptureDependencies(cs, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies));
+  BCK(cudaStreamBeginCaptureToGraph(B->body, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+  body_fn(B->body);
+  BCKCAP(cudaStreamEndCapture(B->body, &body), B->body);
+  return MPFC_OK;
+}
+
 template <int SCH>
 int build_batch_graph(mpfc_batch_s* B) {
   cudaStream_t cs = B->cap;
@@ -638,38 +944,91 @@ int build_batch_graph(mpfc_batch_s* B) {
   BCKCAP(cudaStreamGetCaptureInfo(cs, &st, nullptr, &graph, &deps, nullptr, &ndeps), cs);
   cudaGraphConditionalHandle hnd;
   BCKCAP(cudaGraphConditionalHandleCreate(&hnd, graph, 0, 0), cs);
+  cudaGraphConditionalHandle hnd64 = hnd;
+  if (B->df) BCKCAP(cudaGraphConditionalHandleCreate(&hnd64, graph, 0, 0), cs);
   enqueue_batch_prologue<SCH>(B, cs);
-  enqueue_batch_resnorm<SCH>(B, 0, hnd, 1, cs);
-  BCKCAP(cudaStreamGetCaptureInfo(cs, &st, nullptr, &graph, &deps, nullptr, &ndeps), cs);
-  std::vector<cudaGraphNode_t> dv(deps, deps + ndeps);
-  cudaGraphNodeParams cp = {cudaGraphNodeTypeConditional};
-  cp.conditional.handle = hnd;
-  cp.conditional.type = cudaGraphCondTypeWhile;
-  cp.conditional.size = 1;
-  cudaGraphNode_t cnode;
-  BCKCAP(cudaGraphAddNode(&cnode, graph, dv.data(), nullptr, dv.size(), &cp), cs);
-  cudaGraph_t body = cp.conditional.phGraph_out[0];
-  BCKCAP(cudaStreamUpdateCaptureDependencies(cs, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies), cs);
-  BCKCAP(cudaStreamBeginCaptureToGraph(B->body, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal), cs);
-  enqueue_batch_vcycle<SCH>(B, B->body);
-  enqueue_batch_resnorm<SCH>(B, 1, hnd, 1, B->body);
-  cudaError_t e = cudaStreamEndCapture(B->body, &body);
-  if (e != cudaSuccess) {
-    mpfc_set_cuda_error(e, "cudaStreamEndCapture(batch WHILE body)", __FILE__, __LINE__);
-    mpfc_abort_capture(B->body);
+  int rc = MPFC_OK;
+  if (B->df) {
+    enqueue_batch_df_defect<SCH, true>(B, hnd, hnd64, cs);
+    rc = capture_loop(B, hnd, [&](cudaStream_t s) {
+      enqueue_batch_df_vcycle<SCH>(B, s);
+      enqueue_batch_df_defect<SCH, false>(B, hnd, hnd64, s);
+    });
+  } else {
+    enqueue_batch_resnorm<SCH>(B, 0, hnd, 1, cs);
+  }
+  // FP64 V-cycles: every instance, or those that left the correction form's range
+  if (rc == MPFC_OK)
+    rc = capture_loop(B, hnd64, [&](cudaStream_t s) {
+      if (B->df) kb_take64<<<(B->count + 127) / 128, 128, 0, s>>>(B->d_ctl, B->d_glob, B->count);
+      enqueue_batch_vcycle<SCH>(B, s);
+      enqueue_batch_resnorm<SCH>(B, 1, hnd64, 1, s);
+    });
+  if (rc != MPFC_OK) {
     mpfc_abort_capture(cs);
-    return MPFC_ERR_CUDA;
+    return rc;
   }
   enqueue_batch_commit<SCH>(B, cs);
   BCK(cudaStreamEndCapture(cs, &graph));
   cudaGraphExec_t exec;
-  e = cudaGraphInstantiate(&exec, graph, 0);
+  const cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
   cudaGraphDestroy(graph);
   if (e != cudaSuccess) {
     mpfc_set_cuda_error(e, "cudaGraphInstantiate(batch step graph)", __FILE__, __LINE__);
     return MPFC_ERR_CUDA;
   }
   B->exec[SCH - 1] = exec;
+  return MPFC_OK;
+}
+
+// The levels' coefficients, whether the batch runs in correction form (every instance has at
+// least two levels and coefficients in its range), and its tail: the last levels of every
+// instance, of at most kTailCells cells each, in one CTA per instance (as many as all instances
+// have).  A step of 16 instances (128^2 to 1024^2): 5.20 ms, against 5.26 with tails from 16^2
+// and 5.41 with the coarsest solve alone (FP64 V-cycles: 8.59).
+constexpr int kTailCells = 32 * 32;
+int plan_df(mpfc_batch_s* B, std::vector<DPar> (&pars)[2]) {
+  B->df = true;
+  B->tail = kDfTailMax;
+  for (int s = 0; s < 2; ++s) {
+    B->coef[s].assign((size_t)B->count * kMaxLevels, Coef{});
+    DPar zero;
+    memset(&zero, 0, sizeof(zero));
+    pars[s].assign((size_t)B->count * kMaxLevels, zero);
+  }
+  for (int i = 0; i < B->count; ++i) {
+    B->df = B->df && B->nlev[i] >= 2;
+    int t = 1;
+    while (t < B->nlev[i]) {
+      const Lev& L = B->lev[(size_t)i * kMaxLevels + B->nlev[i] - 1 - t];
+      if ((long long)L.m * L.n > kTailCells) break;
+      ++t;
+    }
+    B->tail = std::min(B->tail, t);
+    for (int s = 0; s < 2; ++s)
+      for (int l = 0; l < B->nlev[i]; ++l) {
+        const size_t id = (size_t)i * kMaxLevels + l;
+        B->coef[s][id] = mpfc_coef(&B->each[i], s + 1, B->lev[id].h, 4);
+        B->df = B->df && df_coef_ok(B->coef[s][id]);
+        pars[s][id].L = B->dlev[id];
+        pars[s][id].k = pars[s][id].kb = df_coef_of(B->coef[s][id], s + 1, B->coef[s][id]);
+      }
+  }
+  size_t smem = 0;
+  for (int i = 0; i < B->count; ++i) {
+    const Lev* lv = B->lev.data() + (size_t)i * kMaxLevels;
+    const size_t gc = (size_t)lv[B->nlev[i] - 1].m * lv[B->nlev[i] - 1].n;
+    size_t need = coarse_df_smem((int)gc);
+    if (B->tail >= 2) {
+      size_t cells = 0;
+      for (int l = B->nlev[i] - B->tail; l < B->nlev[i]; ++l) cells += (size_t)lv[l].m * lv[l].n;
+      need = sizeof(float2) * (gc * gc + (need + 7) / 8 + 7 * cells);
+    }
+    smem = std::max(smem, need);
+  }
+  B->tail_smem = smem;
+  BCK(cudaFuncSetAttribute(kb_df_tail<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDfTailSmem));
+  BCK(cudaFuncSetAttribute(kb_df_tail<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDfTailSmem));
   return MPFC_OK;
 }
 
@@ -720,19 +1079,16 @@ extern "C" int mpfc_batch_create(int count, const mpfc_params* each, void* d_wor
     }
     B->tile_x.assign(B->GL, 32);
     B->tile_y.assign(B->GL, 8);
-    for (int s = 0; s < 2; ++s) {
-      B->coef[s].assign((size_t)count * kMaxLevels, Coef{});
-      B->src[s].resize(count);
-    }
+    for (int s = 0; s < 2; ++s) B->src[s].resize(count);
+    std::vector<DPar> pars[2];
+    rc = plan_df(B, pars);
+    if (rc != MPFC_OK) break;
     std::vector<long long> k3off(count);
     std::vector<double> inv_s(count);
     std::vector<float> K3all[2];
     long long k3tot = 0;
     for (int i = 0; i < count; ++i) {
       const mpfc_params& p = each[i];
-      for (int s = 0; s < 2; ++s)
-        for (int l = 0; l < B->nlev[i]; ++l)
-          B->coef[s][(size_t)i * kMaxLevels + l] = mpfc_coef(&p, s + 1, B->lev[(size_t)i * kMaxLevels + l].h, 4);
       for (int s = 0; s < 2; ++s) {
         SourceArgs& A = B->src[s][i];
         A.phik = B->state[3 * i];
@@ -771,6 +1127,8 @@ extern "C" int mpfc_batch_create(int count, const mpfc_params* each, void* d_wor
         (e = cudaMemcpyAsync(B->d_nlev, B->nlev.data(), sizeof(int) * count, cudaMemcpyHostToDevice, s)) ||
         (e = cudaMemcpyAsync(B->d_K3off, k3off.data(), sizeof(long long) * count, cudaMemcpyHostToDevice, s)) ||
         (e = cudaMemcpyAsync(B->d_inv_s, inv_s.data(), sizeof(double) * count, cudaMemcpyHostToDevice, s)) ||
+        (e = cudaMemcpyAsync(B->d_par[0], pars[0].data(), sizeof(DPar) * pars[0].size(), cudaMemcpyHostToDevice, s)) ||
+        (e = cudaMemcpyAsync(B->d_par[1], pars[1].data(), sizeof(DPar) * pars[1].size(), cudaMemcpyHostToDevice, s)) ||
         (e = cudaMemcpyAsync(B->d_state, B->state.data(), sizeof(double*) * 3 * count, cudaMemcpyHostToDevice, s)) ||
         (e = cudaMemcpyAsync(B->d_ctl, c0.data(), sizeof(BCtl) * count, cudaMemcpyHostToDevice, s)) ||
         (e = cudaMemcpyAsync(B->d_glob, &g0, sizeof(g0), cudaMemcpyHostToDevice, s)) ||
@@ -891,7 +1249,12 @@ extern "C" int mpfc_batch_time_smooth(mpfc_batch_t* B, int scheme, int level, in
     BCK(cudaEventRecord(e0, B->stream));
     for (int r = 0; r < reps; ++r)
       for (int color = 0; color < 2; ++color) {
-        if (scheme == 1)
+        if (B->df) {
+          const int tx = B->tile_x[level], ty = B->tile_y[level];
+          auto kern = scheme == 1 ? kb_df_half<1, kGen, false> : kb_df_half<2, kGen, false>;
+          kern<<<grid_for_items(n), half_block(tx, ty), 0, B->stream>>>(it, n, B->d_par[scheme - 1], B->d_lev, B->d_ctl,
+                                                                      color, tx, ty);
+        } else if (scheme == 1)
           kb_smooth<1><<<grid_for_items(n), blk, 0, B->stream>>>(it, n, B->d_lev, B->d_coef[0], B->d_ctl, color);
         else
           kb_smooth<2><<<grid_for_items(n), blk, 0, B->stream>>>(it, n, B->d_lev, B->d_coef[1], B->d_ctl, color);

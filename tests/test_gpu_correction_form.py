@@ -81,3 +81,59 @@ def test_coefficients_outside_the_range_take_the_fp64_cycle(mp, oracle_mod):
     cycles the oracle itself is within 1.6e-13 of its run in extended precision."""
     g = lockstep(mp, oracle_mod, 128, 64, 1, 8, h=1e-5, s=1e-10)
     assert g.launch_counts(1)[1] == 3 * 11 + 2
+
+
+def _follow_singles(mp, cfgs, scheme, steps=2, **kw):
+    ps = [mp.default_params(h=0.5, m=m, n=n, dt=s, **kw) for m, n, s, _ in cfgs]
+    b = mp.BatchSolver(ps)
+    singles = []
+    for i, (p, (m, n, s, amp)) in enumerate(zip(ps, cfgs)):
+        phi0 = inputs.noise_field(m, n, 0.07, 0.05, 30 + i)
+        if amp > 1:
+            phi0 = amp * (1.0 + 0.01 * inputs.noise_field(m, n, 0.0, 1.0, 30 + i))
+        b.set_state(i, phi0)
+        g = mp.Solver(p)
+        g.set_state(phi0)
+        singles.append(g)
+    for step in range(steps):
+        rc, st = b.step_cycles(scheme, 4)
+        assert rc == 0
+        for i, g in enumerate(singles):
+            g.step_cycles(scheme, 4)
+            a, ref = b.get_state(i)[0], g.get_state()[0]
+            assert np.abs(a - ref).max() <= 1e-12 * np.abs(ref).max(), (step, i)
+
+
+# 1e-12: the bar of the batch against single instances (tests/test_gpu_batch.py)
+@pytest.mark.parametrize("scheme", [1, 2])
+@pytest.mark.parametrize("nu1,nu2", [(2, 2), (0, 2), (2, 0), (1, 3)])
+def test_batches_of_uneven_depth(mp, scheme, nu1, nu2):
+    """Instances of two levels (all of them in the tail) beside deeper ones, with each coarsest
+    grid's size; without the small ones, a tail of four levels; and a single-level instance,
+    with which the whole batch keeps the FP64 V-cycle."""
+    small = [(8, 8, 0.05, 1.0), (12, 20, 0.05, 1.0)]
+    large = [(128, 192, 0.05, 1.0), (96, 160, 0.02, 1.0), (128, 32, 0.05, 1.0)]
+    for cfgs in (small + large, large, large[1:] + [(8, 6, 0.05, 1.0)]):
+        _follow_singles(mp, cfgs, scheme, nu1=nu1, nu2=nu2)
+
+
+def test_batch_instance_outside_the_range(mp):
+    """One instance of |phi| near 2^21 takes the FP64 loop (the oracle's run of it converges)."""
+    _follow_singles(mp, [(64, 64, 0.05, 1.0), (96, 64, 1e-5, 2.0 ** 21), (128, 128, 0.05, 1.0)], 1)
+
+
+@pytest.mark.parametrize("tx,ty", [(1024, 1), (1, 1024), (64, 16), (32, 2)])
+def test_batch_tiles_larger_than_a_block(mp, tx, ty):
+    ps = [mp.default_params(h=0.5, m=m, n=n, dt=0.05) for m, n in ((128, 192), (96, 160))]
+    out = []
+    for tile in (None, (tx, ty)):
+        b = mp.BatchSolver(ps)
+        for i, p in enumerate(ps):
+            b.set_state(i, inputs.noise_field(p.m, p.n, 0.07, 0.05, i))
+        if tile:
+            for level in range(b.levels - 1):
+                b.set_tile(level, *tile)
+        assert b.step(2, 2)[0] == 0
+        out.append([b.get_state(i)[0] for i in range(2)])
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
