@@ -31,6 +31,11 @@ int mpfc_probe_rcp(const double* d_x, double* d_out, int n, void* cuda_stream);
  * `cuda_stream`. */
 int mpfc_probe_convert(const double* d_x, float* d_rn, float* d_trunc, double* d_back, int n, void* cuda_stream);
 
+/* Applies the integer-pipe five-point sum f0 + f1 + f2 + f3 - 4 f4 (the Laplacian of the
+ * residual, the source and the guess) to n groups of five consecutive device doubles, for
+ * tests of its error bound.  Asynchronous on `cuda_stream`. */
+int mpfc_probe_lap5(const double* d_f, double* d_out, int n, void* cuda_stream);
+
 /* Evaluates the convolution kernels' GELU and its derivative (erf by the rational
  * approximation of Abramowitz & Stegun 7.1.26, absolute error <= 1.5e-7) on n device
  * floats: d_g = GELU(z), d_dg = GELU'(z).  For tests against the exact functions.

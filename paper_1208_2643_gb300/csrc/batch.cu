@@ -376,7 +376,7 @@ __global__ void kb_df_apply(const BItem* __restrict__ items, int n, const DPar* 
 // kb_resnorm with the correction form's inputs (df_defect_cell).  An instance with a value
 // outside the form's range stops here and continues in the FP64 loop (kb_take64).
 template <int SCH, bool MODE0>
-__global__ void __launch_bounds__(256) kb_df_defect(const BItem* __restrict__ items, int n, const int* __restrict__ ibeg,
+__global__ void __launch_bounds__(kPTX / 2 * kPTY) kb_df_defect(const BItem* __restrict__ items, int n, const int* __restrict__ ibeg,
                                                     int count, const Lev* __restrict__ levs,
                                                     const Coef* __restrict__ coefs, const DPar* __restrict__ pars, BCtl* ctl,
                                                     BGlobal* glob, double* partials, int zero,
@@ -389,12 +389,15 @@ __global__ void __launch_bounds__(256) kb_df_defect(const BItem* __restrict__ it
     if (MODE0 ? !ctl[w.inst].halted : (bool)ctl[w.inst].active) {
       const int id = w.inst * kMaxLevels;
       const Lev& L = levs[id];
-      const int i = w.x0 + threadIdx.x, j = w.y0 + threadIdx.y;
-      if (i < L.m && j < L.n) {
+      const int x = (w.x0 >> 1) + threadIdx.x, j = w.y0 + threadIdx.y;   // the item's pairs of cells
+      DSum sum{0.0, df{0.f, 0.f}};
+      const float scale = MODE0 ? 1.0f : df_norm_scale(ctl[w.inst].res);
+      if (x < (L.m >> 1) && j < L.n) {
         bool bad = false;
-        v = df_defect_cell<SCH, MODE0, true>(L, coefs[id], pars[id], i, j, zero, bad);
+        df_defect_pair<SCH, MODE0, true>(L, coefs[id], pars[id], x, j, zero, scale, sum, bad);
         if (bad) atomicOr(&ctl[w.inst].range, 1);
       }
+      v = df_thread_sum<MODE0>(sum, scale);
     }
     const double tot = block_total2d(v, red);
     if (threadIdx.x == 0 && threadIdx.y == 0) partials[it] = tot;
@@ -868,7 +871,7 @@ void enqueue_batch_df_vcycle(mpfc_batch_s* B, cudaStream_t s) {
 template <int SCH, bool MODE0>
 void enqueue_batch_df_defect(mpfc_batch_s* B, cudaGraphConditionalHandle hnd, cudaGraphConditionalHandle hnd64,
                              cudaStream_t s) {
-  kb_df_defect<SCH, MODE0><<<grid_for_items(B->fin_cnt), dim3(kPTX, kPTY), 0, s>>>(
+  kb_df_defect<SCH, MODE0><<<grid_for_items(B->fin_cnt), dim3(kPTX / 2, kPTY), 0, s>>>(
       B->d_items + B->fin_off, B->fin_cnt, B->d_ibeg, B->count, B->d_lev, B->d_coef[SCH - 1], B->d_par[SCH - 1], B->d_ctl,
       B->d_glob, B->d_partials, B->p0.nu1 == 0, hnd, hnd64);
 }

@@ -69,6 +69,17 @@ __device__ __forceinline__ df gquot(df p, df pb, df pk) {
   return scale2(sum3u(t, sqr(pb), sqr(pk)), 0.25f);
 }
 
+__device__ __forceinline__ df mul3(df a) {
+  const float h = fmul(3.0f, a.h);
+  return df{h, __fmaf_rn(3.0f, a.l, __fmaf_rn(3.0f, a.h, -h))};
+}
+// g'(p): 3 p^2, or (3 p^2 + 2 p pk + pk^2) / 4 summed as (2 p^2 + (p + pk)^2) / 4
+template <int SCH>
+__device__ __forceinline__ df df_dg(df p, df pk) {
+  if (SCH == 1) return mul3(sqr(p));
+  return scale2(addu(scale2(sqr(p), 2.0f), sqr(add(p, pk))), 0.25f);
+}
+
 // How much of d is still zero in a level's first sweep: kGen nothing, kOwn the cell's own
 // value (first black half sweep), kAll everything (first red half sweep).
 constexpr int kGen = 0, kOwn = 1, kAll = 2;
@@ -99,11 +110,9 @@ __device__ __forceinline__ void df_update(const DCoef& K, df Lp, df Lm, df Lk, D
   df q, Qq;
   if (SCH == 1) {
     q = sqr(p);
-    Qq = add(mk(K.Q0), df{fmul(3.0f, q.h), __fmaf_rn(3.0f, q.l, __fmaf_rn(3.0f, q.h, -fmul(3.0f, q.h)))});
+    Qq = add(mk(K.Q0), mul3(q));
   } else {
-    // g' = (3 p^2 + 2 p pk + pk^2) / 4 = (p (p + pk) + (p + pk)^2 / 2 ... ) summed as 2 p^2 + (p + pk)^2
-    q = scale2(addu(scale2(sqr(p), 2.0f), sqr(add(p, c.pk))), 0.25f);
-    q = add(q, c.W);
+    q = add(df_dg<2>(p, c.pk), c.W);
     Qq = add(mk(K.Q0), q);
   }
   const df wr = rcp(add(mk(K.D0w), mulu(mk(K.aq), q)));

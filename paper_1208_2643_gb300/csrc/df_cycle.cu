@@ -34,17 +34,20 @@ struct DefectArgs {
 };
 
 template <int SCH, bool MODE0, bool FIRST>
-__global__ void __launch_bounds__(256) k_df_defect(const __grid_constant__ DefectArgs A) {
+__global__ void __launch_bounds__(256, 5) k_df_defect(const __grid_constant__ DefectArgs A) {
   pdl_enter();
-  double v[1] = {0.0};
+  DSum sum{0.0, df{0.f, 0.f}};
+  const float scale = MODE0 ? 1.0f : df_norm_scale(A.ctl->res);
   bool bad = false;
-  const int G = A.L.m * A.L.n;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < G; t += gridDim.x * blockDim.x)
-    v[0] += df_defect_cell<SCH, MODE0, FIRST>(A.L, A.k, A.P, t % A.L.m, t / A.L.m, A.zero, bad);
+  const int half = A.L.m >> 1;
+  for (int j = blockIdx.y * blockDim.y + threadIdx.y; j < A.L.n; j += gridDim.y * blockDim.y)
+    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < half; x += gridDim.x * blockDim.x)
+      df_defect_pair<SCH, MODE0, FIRST>(A.L, A.k, A.P, x, j, A.zero, scale, sum, bad);
+  double v[1] = {df_warp_sum<MODE0>(sum, scale)};
   if (bad) atomicOr(&A.ctl->range, 1);
-  if (!grid_sum<1>(v, A.partials, &A.ctl->counter)) return;
+  if (!grid_sum<1, true>(v, A.partials, &A.ctl->counter)) return;
   Ctl* ctl = A.ctl;
-  const double res = sqrt(v[0] / (3.0 * (double)G));
+  const double res = sqrt(v[0] / (3.0 * (double)(A.L.m * A.L.n)));
   const bool go = resnorm_next(ctl, res, A.mode);
   // residuals this small would lose the low parts' range
   const int range = *(volatile int*)&ctl->range | (go && res < kDfMinResidual);
@@ -263,7 +266,7 @@ void defect(mpfc_s* H, int mode, cudaGraphConditionalHandle hnd, int set_cond, c
   A.mode = mode;
   A.set_cond = set_cond;
   A.zero = H->p.nu1 == 0;
-  const dim3 g(mpfc_reduce_blocks((size_t)H->p.m * H->p.n)), b(256);
+  const dim3 g = pair_grid(H->p.m, H->p.n), b(32, 8);
   // the tail expects its first red sweep done, also where the finest level is in it
   const bool first = !df_unfused(H) || df_tail_first(H) == 0;
   if (mode == 0) {

@@ -15,57 +15,105 @@ __device__ __forceinline__ bool df_out_of_range(double x, int e) {
   return (((unsigned)__double2hiint(x) >> 20) & 0x7FFu) >= 1023u + e;
 }
 
-// FP64 residual of the iterate at cell (i, j): rho as float-float planes, p0 = phi; returns the
-// sum of squares and sets `bad` where a value is outside the range the form covers.  MODE0, right
-// after the guess: rows 2 and 3 hold by construction (k_guess_kappa, k_guess_mu), so
-// rho2 = rho3 = 0; phi^k is split too (scheme 2).  FIRST: the first red half sweep on the values
-// in registers; zero: no pre-smoothing, the correction starts at zero.
+// A thread's sum of squared residuals: FP64 (after the guess, where no norm is known to scale
+// by), or float-float of values scaled by a power of two near the inverse of the last norm (a
+// norm cannot fall by 2^60 or grow by 2^50 in one cycle).  The float-float form spares three
+// FP64 multiply-adds a cell and the FP64 additions of the warp's reduction.
+struct DSum {
+  double d;
+  df f;
+};
+__device__ __forceinline__ float df_norm_scale(double res) {
+  const unsigned e = f64_exp(res);
+  return (e < 1023u - 100u || e > 1023u + 100u) ? 1.0f : __uint_as_float((127u + 1023u - e) << 23);
+}
+__device__ __forceinline__ df df_squares(df a, df b, df c, float scale) {
+  return norm(sum3u(sqr(scale2(a, scale)), sqr(scale2(b, scale)), sqr(scale2(c, scale))));
+}
+// One thread's sum in FP64.
+template <bool FP64>
+__device__ __forceinline__ double df_thread_sum(const DSum& s, float scale) {
+  if (FP64) return s.d;
+  const double inv = (double)__uint_as_float((254u << 23) - __float_as_uint(scale));   // 1 / scale
+  return df_to_f64(s.f) * inv * inv;
+}
+// The warp's total, valid in lane 0 (blocks 32 threads wide).
+template <bool FP64>
+__device__ __forceinline__ double df_warp_sum(const DSum& s, float scale) {
+  if (FP64) {
+    double v = s.d;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    return v;
+  }
+  df f = s.f;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    f = add(f, df{__shfl_down_sync(0xffffffffu, f.h, o), __shfl_down_sync(0xffffffffu, f.l, o)});
+  return df_thread_sum<false>(DSum{0.0, f}, scale);
+}
+
+// FP64 residual of the iterate at the cells (2x, j) and (2x + 1, j): rho as float-float planes,
+// p0 = phi; adds the squares to `sum` and sets `bad` where a value is outside the range the form
+// covers.  MODE0, right after the guess: rows 2 and 3 hold by construction (k_guess_kappa,
+// k_guess_mu), so rho2 = rho3 = 0; phi^k is split too (scheme 2).  FIRST: the first red half
+// sweep on the values in registers (one of the two cells is red, so every lane has one); zero: no
+// pre-smoothing, the correction starts at zero.
 template <int SCH, bool MODE0, bool FIRST>
-__device__ __forceinline__ double df_defect_cell(const Lev& L, const Coef& k, const DPar& P, int i, int j, int zero,
-                                                 bool& bad) {
+__device__ __forceinline__ void df_defect_pair(const Lev& L, const Coef& k, const DPar& P, int x, int j, int zero,
+                                               float scale, DSum& sum, bool& bad) {
   const DLev& D = P.L;
-  const int t = j * L.m + i;
-  double a, b = 0.0, c = 0.0, v;
-  if (MODE0) {
-    a = resid1_at(L, k, i, j);
-    v = a * a;
-  } else {
-    resid_at<SCH>(L, k, i, j, a, b, c);
-    v = fma(a, a, fma(b, b, c * c));
-  }
-  const double p = L.phi[t];
-  bad |= df_out_of_range(p, 20) | df_out_of_range(a, 40) | df_out_of_range(b, 40) | df_out_of_range(c, 40);
-  DCell q;
-  q.rho1 = df_of(a);
-  q.rho2 = MODE0 ? df{0.f, 0.f} : df_of(b);
-  q.rho3 = MODE0 ? df{0.f, 0.f} : df_of(c);
-  q.pb = df_of(p);
-  q.pk = q.W = df{0.f, 0.f};
-  const size_t id = dindex(D, i, j);
-  D.r[0][id] = f2(q.rho1);
-  D.r[1][id] = f2(q.rho2);
-  D.r[2][id] = f2(q.rho3);
-  D.pb[id] = f2(q.pb);
+  PairResid R;
+  resid_pair<SCH, MODE0>(L, k, x, j, R);
   if (SCH == 2 && MODE0) {
-    q.pk = df_of(L.pk[t]);
-    D.pk[id] = f2(q.pk);
+    const double2 pk = ld2(L.pk + (size_t)j * L.m + 2 * x);
+    R.pk[0] = pk.x;
+    R.pk[1] = pk.y;
   }
-  if (zero) {
-    const float2 z = make_float2(0.f, 0.f);
-    D.d[0][id] = z;
-    D.d[1][id] = z;
-    D.d[2][id] = z;
-  } else if (FIRST && !((i + j) & 1)) {
-    if (SCH == 2 && !MODE0) q.pk = ldd(D.pk + id);
-    if (SCH == 2 && D.W) q.W = df_of(D.W[t]);
-    const df z{0.f, 0.f};
-    if (D.nyn && (j == 0 || j == D.n - 1)) df_update<SCH, kAll>(P.kb, z, z, z, q);
-    else df_update<SCH, kAll>(P.k, z, z, z, q);
-    D.d[0][id] = f2(q.p);
-    D.d[1][id] = f2(q.m);
-    D.d[2][id] = f2(q.k);
+  const size_t red = (size_t)j * (D.m >> 1) + x, black = red + dplane(D);
+  const int qr = j & 1;   // which of the two is red
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {   // the red cell, the black cell
+    const bool second = c == 0 ? qr != 0 : qr == 0;
+    const double a = second ? R.a[1] : R.a[0], p = second ? R.p[1] : R.p[0];
+    bad |= df_out_of_range(p, 20) | df_out_of_range(a, 40);
+    DCell q;
+    q.rho1 = df_of(a);
+    q.rho2 = q.rho3 = q.pk = q.W = df{0.f, 0.f};
+    q.pb = df_of(p);
+    if (MODE0) {
+      sum.d = fma(a, a, sum.d);
+    } else {
+      const double b = second ? R.b[1] : R.b[0], d = second ? R.c[1] : R.c[0];
+      bad |= df_out_of_range(b, 40) | df_out_of_range(d, 40);
+      q.rho2 = df_of(b);
+      q.rho3 = df_of(d);
+      sum.f = add(sum.f, df_squares(q.rho1, q.rho2, q.rho3, scale));
+    }
+    const size_t id = c == 0 ? red : black;
+    D.r[0][id] = f2(q.rho1);
+    D.r[1][id] = f2(q.rho2);
+    D.r[2][id] = f2(q.rho3);
+    D.pb[id] = f2(q.pb);
+    if (SCH == 2 && (MODE0 || (FIRST && c == 0))) {
+      q.pk = df_of(second ? R.pk[1] : R.pk[0]);
+      if (MODE0) D.pk[id] = f2(q.pk);
+    }
+    if (zero) {
+      const float2 z = make_float2(0.f, 0.f);
+      D.d[0][id] = z;
+      D.d[1][id] = z;
+      D.d[2][id] = z;
+    } else if (FIRST && c == 0) {
+      if (SCH == 2 && D.W) q.W = df_of(D.W[(size_t)j * D.m + 2 * x + qr]);
+      const df z{0.f, 0.f};
+      if (D.nyn && (j == 0 || j == D.n - 1)) df_update<SCH, kAll>(P.kb, z, z, z, q);
+      else df_update<SCH, kAll>(P.k, z, z, z, q);
+      D.d[0][id] = f2(q.p);
+      D.d[1][id] = f2(q.m);
+      D.d[2][id] = f2(q.k);
+    }
   }
-  return v;
 }
 
 // ---------------------------------------------------------------------------

@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "int_lap.cuh"
 #include "mpfc_common.cuh"
 
 namespace mpfc {
@@ -99,12 +100,16 @@ __device__ __forceinline__ df lap5(df w, df e, df s, df n, df c) {
 __device__ __forceinline__ df df_of(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const unsigned int hi = (unsigned int)(b >> 32), eb = (hi >> 20) & 0x7FFu;
-  const float h = f64_to_f32_trunc(x);
-  if (eb - (1023u - 74u) >= 174u) return df{h, 0.0f};
+  if (eb - (1023u - 74u) >= 174u) {
+    if ((b << 1) == 0ull) return df{0.0f, 0.0f};
+    return df{f64_to_f32_trunc(x), 0.0f};
+  }
+  const unsigned int sg = hi & 0x80000000u, ef = (eb - 1023u + 127u) << 23;
   // low 29 bits times 2^(e - 52), with the sign of x
-  const float sc = __uint_as_float((hi & 0x80000000u) | ((eb - 1023u + 127u - 52u) << 23));
-  return df{h, fmul(__uint2float_rn((unsigned int)b & 0x1FFFFFFFu), sc)};
+  return df{__uint_as_float(sg | ef | ((unsigned int)(b >> 29) & 0x7FFFFFu)),
+            fmul(__uint2float_rn((unsigned int)b & 0x1FFFFFFFu), __uint_as_float(sg | (ef - (52u << 23))))};
 }
+
 // float-float -> binary64 (exact where h and l span at most 53 bits).
 __device__ __forceinline__ double df_to_f64(df a) { return f32_to_f64(a.h) + f32_to_f64(a.l); }
 

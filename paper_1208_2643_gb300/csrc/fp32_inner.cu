@@ -20,6 +20,7 @@
 
 #include <vector>
 
+#include "df_kernels.cuh"
 #include "fp64_kernels.cuh"
 #include "mpfc_internal.h"
 
@@ -55,35 +56,53 @@ dim3 grid_of(int X, int Y) { return dim3((X + kBlk.x - 1) / kBlk.x, (Y + kBlk.y 
 
 // ---------------------------------------------------------------------------
 // FP64 defect: r = S - N(u) and q = gam + g'(phi) as FP32 inputs of the inner solve,
-// e = 0, and the scaled residual norm with the outer loop decision.
+// e = 0, and the scaled residual norm with the outer loop decision.  Bound by the FP64 pipe
+// (8 instructions a cell in scheme 1, the Laplacians being integer sums, lap5_f64); the
+// linearisation and, after the first cycle, the squares are float-float (as in
+// df_defect_cell): @D@ us at 1024^2, 75 with all of it in FP64.
 // ---------------------------------------------------------------------------
 template <int SCH>
-__global__ void __launch_bounds__(256) k_defect(Lev L, Coef k, Lev32 E, Ctl* ctl, double* partials, int mode,
+__global__ void __launch_bounds__(256, 5) k_defect(Lev L, Coef k, Lev32 E, Ctl* ctl, double* partials, int mode,
                                                 cudaGraphConditionalHandle hnd, int set_cond) {
   pdl_enter();
-  double v[1] = {0.0};
-  int G = L.m * L.n;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < G; t += gridDim.x * blockDim.x) {
-    int i = t % L.m, j = t / L.m;
-    double a, b, c;
-    resid_at<SCH>(L, k, i, j, a, b, c);
-    v[0] = fma(a, a, fma(b, b, fma(c, c, v[0])));
-    double p = L.phi[t];
-    double pk = (SCH == 2) ? L.pk[t] : 0.0;
-    // defect and linearisation handed to the FP32 solve, rounded to nearest (a
-    // non-finite defect stays non-finite, so the residual test above sees it)
-    E.r1[t] = f64_to_f32_rn(a);
-    E.r2[t] = f64_to_f32_rn(b);
-    E.r3[t] = f64_to_f32_rn(c);
-    // q = gam + g'(phi), plus the pinning weight (Sec. 4.6, scheme 2: gam -> gam + W)
-    const double wq = (SCH == 2 && L.W) ? L.W[t] : 0.0;
-    E.q[t] = f64_to_f32_rn(k.gam + wq + dg_of<SCH>(p, pk));
-    E.ephi[t] = 0.f;
-    E.emu[t] = 0.f;
-    E.eka[t] = 0.f;
-  }
-  if (!grid_sum<1>(v, partials, &ctl->counter)) return;
-  double res = sqrt(v[0] / (3.0 * (double)G));
+  DSum sum{0.0, df{0.f, 0.f}};
+  const float scale = mode == 0 ? 1.0f : df_norm_scale(ctl->res);
+  const df gam = df_of(k.gam);
+  const int half = L.m >> 1;
+  for (int j = blockIdx.y * blockDim.y + threadIdx.y; j < L.n; j += gridDim.y * blockDim.y)
+    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < half; x += gridDim.x * blockDim.x) {
+      PairResid R;
+      resid_pair<SCH, false>(L, k, x, j, R);
+      // defect and linearisation handed to the FP32 solve, rounded to nearest (a
+      // non-finite defect stays non-finite, so the residual test sees it)
+      float o1[2], o2[2], o3[2], oq[2];
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const df r1 = df_of(R.a[c]), r2 = df_of(R.b[c]), r3 = df_of(R.c[c]);
+        if (mode == 0) sum.d = fma(R.a[c], R.a[c], fma(R.b[c], R.b[c], fma(R.c[c], R.c[c], sum.d)));
+        else sum.f = add(sum.f, df_squares(r1, r2, r3, scale));
+        o1[c] = fadd(r1.h, r1.l);
+        o2[c] = fadd(r2.h, r2.l);
+        o3[c] = fadd(r3.h, r3.l);
+        // q = gam + g'(phi), plus the pinning weight (Sec. 4.6, scheme 2: gam -> gam + W)
+        const df p = df_of(R.p[c]);
+        df q = add(gam, df_dg<SCH>(p, SCH == 2 ? df_of(R.pk[c]) : p));
+        if (SCH == 2 && L.W) q = add(q, df_of(R.W[c]));
+        oq[c] = fadd(q.h, q.l);
+      }
+      const size_t id = (size_t)j * L.m + 2 * x;
+      auto put = [&](float* f, float a, float b) { *reinterpret_cast<float2*>(f + id) = make_float2(a, b); };
+      put(E.r1, o1[0], o1[1]);
+      put(E.r2, o2[0], o2[1]);
+      put(E.r3, o3[0], o3[1]);
+      put(E.q, oq[0], oq[1]);
+      put(E.ephi, 0.f, 0.f);
+      put(E.emu, 0.f, 0.f);
+      put(E.eka, 0.f, 0.f);
+    }
+  double v[1] = {mode == 0 ? df_warp_sum<true>(sum, scale) : df_warp_sum<false>(sum, scale)};
+  if (!grid_sum<1, true>(v, partials, &ctl->counter)) return;
+  double res = sqrt(v[0] / (3.0 * (double)(L.m * L.n)));
   int cond;
   if (mode == 0) {
     ctl->res0 = res;
@@ -1051,12 +1070,12 @@ void enqueue_inner_vcycle(mpfc_s* H, int scheme, cudaStream_t s) {
 
 void enqueue_defect(mpfc_s* H, int scheme, int mode, cudaGraphConditionalHandle hnd, int set_cond, cudaStream_t s) {
   const Lev& L0 = H->lev[0];
-  int blocks = mpfc_reduce_blocks((size_t)L0.m * L0.n);
+  const dim3 g = pair_grid(L0.m, L0.n), b(32, 8);
   if (scheme == 1)
-    mpfc_launch(H->shape, k_defect<1>, dim3(blocks), dim3(256), 0, s, L0, H->coef[0][0], H->lev32[0], H->ctl,
+    mpfc_launch(H->shape, k_defect<1>, g, b, 0, s, L0, H->coef[0][0], H->lev32[0], H->ctl,
                 H->partials, mode, hnd, set_cond);
   else
-    mpfc_launch(H->shape, k_defect<2>, dim3(blocks), dim3(256), 0, s, L0, H->coef[1][0], H->lev32[0], H->ctl,
+    mpfc_launch(H->shape, k_defect<2>, g, b, 0, s, L0, H->coef[1][0], H->lev32[0], H->ctl,
                 H->partials, mode, hnd, set_cond);
 }
 

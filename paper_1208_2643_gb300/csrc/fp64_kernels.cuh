@@ -7,6 +7,7 @@
 // on the FP64 instruction count per cell.
 #pragma once
 
+#include "int_lap.cuh"
 #include "mpfc_common.cuh"
 
 namespace mpfc {
@@ -36,7 +37,7 @@ __device__ __forceinline__ void source_cell(const Lev& L, const SourceArgs& A, i
   double ih2 = 1.0 / (L.h * L.h);
   const double* pk = A.phik;
   double p0 = pk[c];
-  double lap_k = ((pk[w] + pk[e]) + (pk[s] + pk[nn]) - 4.0 * p0) * ih2;
+  const double lap_k = lap5_f64(pk[w], pk[e], pk[s], pk[nn], p0) * ih2;
   double q0 = A.phikm1[c];
   if (SCH == 1) {
     L.S1[c] = p0 + A.psi_coef * A.psik[c];
@@ -44,14 +45,12 @@ __device__ __forceinline__ void source_cell(const Lev& L, const SourceArgs& A, i
     L.S3[c] = 0.0;
   } else {
     const double* pm = A.phikm1;
-    // phitilde = (3 phik - phikm1)/2 at the five points, then Delta_h of it
-    double t0 = 0.5 * (3.0 * p0 - q0);
-    double tw = 0.5 * (3.0 * pk[w] - pm[w]), te = 0.5 * (3.0 * pk[e] - pm[e]);
-    double ts = 0.5 * (3.0 * pk[s] - pm[s]), tn = 0.5 * (3.0 * pk[nn] - pm[nn]);
-    double lap_t = ((tw + te) + (ts + tn) - 4.0 * t0) * ih2;
+    // 2 Delta_h phitilde, phitilde = (3 phik - phikm1)/2: 3 Delta_h phik - Delta_h phikm1
+    const double lap_m = lap5_f64(pm[w], pm[e], pm[s], pm[nn], q0) * ih2;
+    const double lap_t2 = fma(3.0, lap_k, -lap_m);
     L.S1[c] = p0 + A.psi_coef * A.psik[c];
     // pinning (Sec. 4.6): 2 W (phi^{k+1/2} - phihat) minus its part W phi in N gives W (phi^k - 2 phihat)
-    L.S2[c] = A.half_alpha * p0 + 2.0 * lap_t + (A.W ? A.W[c] * (p0 - 2.0 * A.phihat[c]) : 0.0);
+    L.S2[c] = A.half_alpha * p0 + lap_t2 + (A.W ? A.W[c] * (p0 - 2.0 * A.phihat[c]) : 0.0);
     L.S3[c] = 0.5 * lap_k;
   }
   if (A.guess == 0) L.phi[c] = p0;
@@ -73,8 +72,8 @@ __device__ __forceinline__ void guess_kappa_cell(const Lev& L, const Coef& k, in
   int im = wrapm(i - 1, m), ip = wrapm(i + 1, m), jm = ywrap(j - 1, L.n, L.nyn), jp = ywrap(j + 1, L.n, L.nyn);
   size_t c = (size_t)j * m + i;
   const double* f = L.phi;
-  double sum = (f[(size_t)j * m + im] + f[(size_t)j * m + ip]) + (f[(size_t)jm * m + i] + f[(size_t)jp * m + i]);
-  L.ka[c] = L.S3[c] + k.th2 * (sum - 4.0 * f[c]);
+  const double lap = lap5_f64(f[(size_t)j * m + im], f[(size_t)j * m + ip], f[(size_t)jm * m + i], f[(size_t)jp * m + i], f[c]);
+  L.ka[c] = fma(k.th2, lap, L.S3[c]);
 }
 
 static __global__ void k_guess_kappa(Lev L, Coef k) {
@@ -92,11 +91,11 @@ __device__ __forceinline__ void guess_mu_cell(const Lev& L, const Coef& k, int i
   int im = wrapm(i - 1, m), ip = wrapm(i + 1, m), jm = ywrap(j - 1, L.n, L.nyn), jp = ywrap(j + 1, L.n, L.nyn);
   size_t c = (size_t)j * m + i;
   const double* f = L.ka;
-  double sum = (f[(size_t)j * m + im] + f[(size_t)j * m + ip]) + (f[(size_t)jm * m + i] + f[(size_t)jp * m + i]);
-  double p = L.phi[c];
-  double pk = (SCH == 2) ? L.pk[c] : 0.0;
-  double gam = (SCH == 2 && L.W) ? k.gam + L.W[c] : k.gam;   // pinning weight joins gam (Sec. 4.6)
-  L.mu[c] = L.S2[c] + g_of<SCH>(p, pk) + gam * p + k.ih2 * (sum - 4.0 * f[c]);
+  const double lap = lap5_f64(f[(size_t)j * m + im], f[(size_t)j * m + ip], f[(size_t)jm * m + i], f[(size_t)jp * m + i], f[c]);
+  const double p = L.phi[c];
+  const double pk = (SCH == 2) ? L.pk[c] : 0.0;
+  const double gam = (SCH == 2 && L.W) ? k.gam + L.W[c] : k.gam;   // pinning weight joins gam (Sec. 4.6)
+  L.mu[c] = fma(k.ih2, lap, L.S2[c] + fma(gam, p, g_of<SCH>(p, pk)));
 }
 
 template <int SCH>
@@ -123,18 +122,100 @@ __device__ __forceinline__ void resid_at(const Lev& L, const Coef& k, int i, int
   const double* phi = L.phi;
   const double* mu = L.mu;
   const double* ka = L.ka;
-  double p = __ldg(phi + c), u = __ldg(mu + c), v = __ldg(ka + c);
-  double smu = (__ldg(mu + w) + __ldg(mu + e)) + (__ldg(mu + s) + __ldg(mu + nn));
-  double ska = (__ldg(ka + w) + __ldg(ka + e)) + (__ldg(ka + s) + __ldg(ka + nn));
-  double sph = (__ldg(phi + w) + __ldg(phi + e)) + (__ldg(phi + s) + __ldg(phi + nn));
-  double pk = (SCH == 2) ? __ldg(L.pk + c) : 0.0;
+  const double p = __ldg(phi + c), u = __ldg(mu + c), v = __ldg(ka + c);
+  const double lm = lap5_f64(__ldg(mu + w), __ldg(mu + e), __ldg(mu + s), __ldg(mu + nn), u);
+  const double lk = lap5_f64(__ldg(ka + w), __ldg(ka + e), __ldg(ka + s), __ldg(ka + nn), v);
+  const double lp = lap5_f64(__ldg(phi + w), __ldg(phi + e), __ldg(phi + s), __ldg(phi + nn), p);
   // r1 = S1 - phi + c Delta_h mu
-  r1 = fma(k.cmu, fma(-4.0, u, smu), __ldg(L.S1 + c) - p);
+  r1 = fma(k.cmu, lm, __ldg(L.S1 + c) - p);
   // r2 = S2 - mu + g(phi) + gam phi + Delta_h kappa
-  double gam = (SCH == 2 && L.W) ? k.gam + __ldg(L.W + c) : k.gam;
-  r2 = fma(k.ih2, fma(-4.0, v, ska), fma(gam, p, __ldg(L.S2 + c) - u) + g_of<SCH>(p, pk));
+  double t;
+  if (SCH == 1) {
+    t = fma(fma(p, p, k.gam), p, __ldg(L.S2 + c)) - u;
+  } else {
+    const double pk = __ldg(L.pk + c);
+    const double gam = L.W ? k.gam + __ldg(L.W + c) : k.gam;
+    t = fma(0.25 * fma(p, p, pk * pk), p + pk, fma(gam, p, __ldg(L.S2 + c) - u));
+  }
+  r2 = fma(k.ih2, lk, t);
   // r3 = S3 - kappa + theta Delta_h phi
-  r3 = fma(k.th2, fma(-4.0, p, sph), __ldg(L.S3 + c) - v);
+  r3 = fma(k.th2, lp, __ldg(L.S3 + c) - v);
+}
+
+// The residual of the two cells (2x, j) and (2x + 1, j): aligned 16-byte loads of the row
+// pairs (m is even and the planes are 256-byte aligned), and each value's exponent taken once.
+// ROW1: row 1 alone, b and c untouched.
+struct PairResid {
+  double a[2], b[2], c[2], p[2], pk[2], W[2];
+};
+__device__ __forceinline__ double2 ld2(const double* f) { return __ldg(reinterpret_cast<const double2*>(f)); }
+
+struct PairNb {
+  size_t o, s, n, w, e;   // offsets of (2x, j), (2x, j -+ 1), (2x - 1, j) and (2x + 2, j)
+};
+__device__ __forceinline__ PairNb pair_nb(const Lev& L, int x, int j) {
+  const int m = L.m, i = 2 * x;
+  const size_t row = (size_t)j * m;
+  PairNb q;
+  q.o = row + i;
+  q.s = (size_t)ywrap(j - 1, L.n, L.nyn) * m + i;
+  q.n = (size_t)ywrap(j + 1, L.n, L.nyn) * m + i;
+  q.w = row + (i > 0 ? i - 1 : m - 1);
+  q.e = row + (i + 2 < m ? i + 2 : 0);
+  return q;
+}
+__device__ __forceinline__ void pair_lap(const double* f, const PairNb& q, double2 o, double& l0, double& l1) {
+  const double2 s = ld2(f + q.s), n = ld2(f + q.n);
+  l0 = lap5_f64(__ldg(f + q.w), o.y, s.x, n.x, o.x);
+  l1 = lap5_f64(o.x, __ldg(f + q.e), s.y, n.y, o.y);
+}
+
+template <int SCH, bool ROW1>
+__device__ __forceinline__ void resid_pair(const Lev& L, const Coef& k, int x, int j, PairResid& R) {
+  const PairNb q = pair_nb(L, x, j);
+  const double2 p = ld2(L.phi + q.o), u = ld2(L.mu + q.o), S1 = ld2(L.S1 + q.o);
+  R.p[0] = p.x;
+  R.p[1] = p.y;
+  double l0, l1;
+  pair_lap(L.mu, q, u, l0, l1);
+  R.a[0] = fma(k.cmu, l0, S1.x - p.x);
+  R.a[1] = fma(k.cmu, l1, S1.y - p.y);
+  if (ROW1) return;
+  const double2 v = ld2(L.ka + q.o), S2 = ld2(L.S2 + q.o), S3 = ld2(L.S3 + q.o);
+  double g0 = k.gam, g1 = k.gam, t0, t1;
+  if (SCH == 1) {
+    t0 = fma(fma(p.x, p.x, g0), p.x, S2.x) - u.x;
+    t1 = fma(fma(p.y, p.y, g1), p.y, S2.y) - u.y;
+  } else {
+    const double2 pk = ld2(L.pk + q.o);
+    R.pk[0] = pk.x;
+    R.pk[1] = pk.y;
+    if (L.W) {
+      const double2 w = ld2(L.W + q.o);
+      R.W[0] = w.x;
+      R.W[1] = w.y;
+      g0 += w.x;
+      g1 += w.y;
+    }
+    t0 = fma(0.25 * fma(p.x, p.x, pk.x * pk.x), p.x + pk.x, fma(g0, p.x, S2.x - u.x));
+    t1 = fma(0.25 * fma(p.y, p.y, pk.y * pk.y), p.y + pk.y, fma(g1, p.y, S2.y - u.y));
+  }
+  pair_lap(L.ka, q, v, l0, l1);
+  R.b[0] = fma(k.ih2, l0, t0);
+  R.b[1] = fma(k.ih2, l1, t1);
+  pair_lap(L.phi, q, p, l0, l1);
+  R.c[0] = fma(k.th2, l0, S3.x - v.x);
+  R.c[1] = fma(k.th2, l1, S3.y - v.y);
+}
+
+// Launch of a one-sum reduction over the pairs of an m x n level: blocks of 32 x 8 pairs, at
+// most kMaxSums * kMaxPartials of them (one sum may use the whole partials array); kernels
+// stride over what is left.
+inline dim3 pair_grid(int m, int n) {
+  const int most = kMaxSums * kMaxPartials;
+  const int gx = (m / 2 + 31) / 32 < most ? (m / 2 + 31) / 32 : most;
+  const int gy = (n + 7) / 8, cap = most / gx;
+  return dim3(gx, gy < cap ? gy : cap);
 }
 
 template <int SCH>
@@ -714,7 +795,8 @@ __global__ void k_coarse_solve(Lev C, Coef k, const float* __restrict__ K3f) {
 // ---------------------------------------------------------------------------
 template <int NS>
 __device__ __forceinline__ void block_sum(double (&v)[NS], double* red /* NS * 32 */) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const int lane = tid & 31, wid = tid >> 5, nw = (blockDim.x * blockDim.y) >> 5;
 #pragma unroll
   for (int s = 0; s < NS; ++s)
 #pragma unroll
@@ -735,18 +817,32 @@ __device__ __forceinline__ void block_sum(double (&v)[NS], double* red /* NS * 3
 }
 
 // Returns true in the one thread (thread 0 of the last block) that holds the
-// totals in v after the call.
-template <int NS>
+// totals in v after the call.  Blocks and grids of any shape; WARPS: each warp's sum is
+// already in its lane 0 (v of the other lanes is ignored).
+template <int NS, bool WARPS = false>
 __device__ __forceinline__ bool grid_sum(double (&v)[NS], double* partials, unsigned int* counter) {
   __shared__ double red[NS * 32];
   __shared__ bool last;
-  block_sum<NS>(v, red);
-  if (threadIdx.x == 0) {
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x, nth = blockDim.x * blockDim.y;
+  if (WARPS) {
+    // up to eight warps: three additions per block instead of five per warp
+    if ((tid & 31) == 0) red[tid >> 5] = v[0];
+    __syncthreads();
+    if (tid < 32) {
+      double x = tid < (nth >> 5) ? red[tid] : 0.0;
 #pragma unroll
-    for (int s = 0; s < NS; ++s) partials[s * kMaxPartials + blockIdx.x] = v[s];
+      for (int o = 4; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+      v[0] = x;
+    }
+  } else {
+    block_sum<NS>(v, red);
+  }
+  if (tid == 0) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s) partials[s * kMaxPartials + blockIdx.y * gridDim.x + blockIdx.x] = v[s];
     __threadfence();
     unsigned int done = atomicAdd(counter, 1u);
-    last = (done == gridDim.x - 1);
+    last = (done == gridDim.x * gridDim.y - 1);
   }
   __syncthreads();
   if (!last) return false;
@@ -755,10 +851,10 @@ __device__ __forceinline__ bool grid_sum(double (&v)[NS], double* partials, unsi
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
     w[s] = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) w[s] += ((volatile double*)partials)[s * kMaxPartials + b];
+    for (int b = tid; b < (int)(gridDim.x * gridDim.y); b += nth) w[s] += ((volatile double*)partials)[s * kMaxPartials + b];
   }
   block_sum<NS>(w, red);
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     *counter = 0u;
 #pragma unroll
     for (int s = 0; s < NS; ++s) v[s] = w[s];
@@ -799,9 +895,9 @@ __device__ __forceinline__ double resid1_at(const Lev& L, const Coef& k, int i, 
   const int im = wrapm(i - 1, m), ip = wrapm(i + 1, m), jm = ywrap(j - 1, L.n, L.nyn), jp = ywrap(j + 1, L.n, L.nyn);
   const size_t c = (size_t)j * m + i;
   const double* mu = L.mu;
-  const double smu = (__ldg(mu + (size_t)j * m + im) + __ldg(mu + (size_t)j * m + ip)) +
-                     (__ldg(mu + (size_t)jm * m + i) + __ldg(mu + (size_t)jp * m + i));
-  return fma(k.cmu, fma(-4.0, __ldg(mu + c), smu), __ldg(L.S1 + c) - __ldg(L.phi + c));
+  const double lm = lap5_f64(__ldg(mu + (size_t)j * m + im), __ldg(mu + (size_t)j * m + ip), __ldg(mu + (size_t)jm * m + i),
+                             __ldg(mu + (size_t)jp * m + i), __ldg(mu + c));
+  return fma(k.cmu, lm, __ldg(L.S1 + c) - __ldg(L.phi + c));
 }
 
 // Scaled residual norm at the finest level, and the V-cycle loop decision.  R1ONLY:

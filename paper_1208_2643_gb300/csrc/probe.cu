@@ -6,6 +6,7 @@
 #include "../../include/mpfc.h"
 #include "../../include/mpfc_probe.h"
 #include "cnn_math.cuh"
+#include "int_lap.cuh"
 #include "mpfc_common.cuh"
 
 namespace {
@@ -118,5 +119,19 @@ extern "C" int mpfc_probe_gelu8(const float* d_z, float* d_g, int n, void* cuda_
   if (n == 0) return MPFC_OK;
   const int threads = (n + 7) / 8;
   k_gelu8<<<(threads + 255) / 256, 256, 0, (cudaStream_t)cuda_stream>>>(d_z, d_g, n);
+  return cudaGetLastError() == cudaSuccess ? MPFC_OK : MPFC_ERR_CUDA;
+}
+
+namespace {
+__global__ void k_lap5(const double* __restrict__ f, double* __restrict__ out, int n) {
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = mpfc::lap5_f64(f[5 * i], f[5 * i + 1], f[5 * i + 2], f[5 * i + 3], f[5 * i + 4]);
+}
+}  // namespace
+
+extern "C" int mpfc_probe_lap5(const double* d_f, double* d_out, int n, void* cuda_stream) {
+  if (!d_f || !d_out || n < 0) return MPFC_ERR_INVALID;
+  if (n == 0) return MPFC_OK;
+  k_lap5<<<(n + 255) / 256, 256, 0, (cudaStream_t)cuda_stream>>>(d_f, d_out, n);
   return cudaGetLastError() == cudaSuccess ? MPFC_OK : MPFC_ERR_CUDA;
 }
