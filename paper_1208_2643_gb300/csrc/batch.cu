@@ -344,13 +344,13 @@ __global__ void __launch_bounds__(kDfTailThreads, 1) kb_df_tail(const DPar* __re
   df_tail_body<SCH, false>(DTailDim{tail, nu1, nu2, 0}, lv, K3 + K3off[inst], tsm, sl, [] {});
 }
 template <int SCH>
-__global__ void __launch_bounds__(32) kb_df_coarse(const DPar* __restrict__ pars, const int* __restrict__ nlev,
+__global__ void __launch_bounds__(kDfTailThreads) kb_df_coarse(const DPar* __restrict__ pars, const int* __restrict__ nlev,
                                                    const float* __restrict__ K3, const long long* __restrict__ K3off,
                                                    const BCtl* __restrict__ ctl) {
   extern __shared__ float2 tsm[];
   const int inst = blockIdx.x;
   if (!ctl[inst].active) return;
-  coarse_df_warp<SCH>(pars[inst * kMaxLevels + nlev[inst] - 1], K3 + K3off[inst], tsm);
+  coarse_df_block<SCH>(pars[inst * kMaxLevels + nlev[inst] - 1], K3 + K3off[inst], tsm);
 }
 
 // u += d of the instances whose finest level took no final half sweep (it is in the tail, or
@@ -373,7 +373,7 @@ __global__ void kb_df_apply(const BItem* __restrict__ items, int n, const DPar* 
   }
 }
 
-// kb_resnorm with the correction form's inputs (df_defect_cell).  An instance with a value
+// kb_resnorm with the correction form's inputs (df_defect_pair).  An instance with a value
 // outside the form's range stops here and continues in the FP64 loop (kb_take64).
 template <int SCH, bool MODE0>
 __global__ void __launch_bounds__(kPTX / 2 * kPTY) kb_df_defect(const BItem* __restrict__ items, int n, const int* __restrict__ ibeg,
@@ -853,7 +853,7 @@ void enqueue_batch_df_vcycle(mpfc_batch_s* B, cudaStream_t s) {
     kb_df_tail<SCH><<<B->count, kDfTailThreads, B->tail_smem, s>>>(pars, B->d_nlev, B->d_K3[S], B->d_K3off, B->d_ctl,
                                                                  B->tail, p.nu1, p.nu2);
   else
-    kb_df_coarse<SCH><<<B->count, 32, B->tail_smem, s>>>(pars, B->d_nlev, B->d_K3[S], B->d_K3off, B->d_ctl);
+    kb_df_coarse<SCH><<<B->count, kDfTailThreads, B->tail_smem, s>>>(pars, B->d_nlev, B->d_K3[S], B->d_K3off, B->d_ctl);
   for (int gl = gt - 1; gl >= 0; --gl) {
     const int n = B->full_cnt[gl + 1];
     if (n) kb_df_prolong<<<grid_for_items(n), blk2, 0, s>>>(B->d_items + B->full_off[gl + 1], n, pars, B->d_ctl);

@@ -124,10 +124,10 @@ __global__ void k_df_restrict_pk(const double* __restrict__ f, double* __restric
 }
 
 template <int SCH>
-__global__ void __launch_bounds__(32) k_df_coarse(const __grid_constant__ DPar P, const float* __restrict__ K3f) {
+__global__ void __launch_bounds__(kDfTailThreads) k_df_coarse(const __grid_constant__ DPar P, const float* __restrict__ K3f) {
   extern __shared__ float2 csm[];
   pdl_enter();
-  coarse_df_warp<SCH>(P, K3f, csm);
+  coarse_df_block<SCH>(P, K3f, csm);
 }
 
 struct DTailArgs {
@@ -234,7 +234,7 @@ void vcycle(mpfc_s* H, cudaStream_t s) {
       launch_df_tail<SCH>(H, lt, s);
     } else {
       const int G = H->lev[L - 1].m * H->lev[L - 1].n;
-      mpfc_launch(sh, k_df_coarse<SCH>, dim3(1), dim3(32), coarse_df_smem(G), s, dpar(H, SCH, L - 1),
+      mpfc_launch(sh, k_df_coarse<SCH>, dim3(1), dim3(kDfTailThreads), coarse_df_smem(G), s, dpar(H, SCH, L - 1),
                   (const float*)H->K3[SCH - 1]);
     }
   }

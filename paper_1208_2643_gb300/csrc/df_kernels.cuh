@@ -120,10 +120,13 @@ __device__ __forceinline__ void df_defect_pair(const Lev& L, const Coef& k, cons
 // Coarsest grid: Newton on the equation for d_phi with rows 2 and 3 eliminated,
 //   F(d) = d - c L (rho2 + g(p0 + d) - g(p0) + (gam + W) d + L (rho3 + theta L d)) - rho1 = 0,
 // J = K3 - c L diag(gam + W + g'(p0 + d)): the FP64 form's equation (coarse_newton), with
-// F in float-float and the same FP32 linear solves.  Stops once the applied update is below
-// 1e-15 (1 + |p0 + d|_inf), as there, or below 1e-14 |d|_inf, the arithmetic's resolution.
-// One warp; sm: 6 G float2 and the FP32 part.
+// F in float-float and FP32 linear solves.  The applied update is below 1e-15 (1 + |p0 + d|_inf),
+// as there, or below 1e-14 |d|_inf, the arithmetic's resolution, or was predicted to be on
+// the next pass.
 // ---------------------------------------------------------------------------
+constexpr int kDfTailMax = 10;
+constexpr int kDfTailThreads = 512;
+
 __device__ __forceinline__ df nblap_df(const float2* f, int m, int n, int t, int nyn) {
   const int i = t % m, j = t / m;
   return lap5(ldd(f + j * m + wrapm(i - 1, m)), ldd(f + j * m + wrapm(i + 1, m)), ldd(f + ywrap(j - 1, n, nyn) * m + i),
@@ -132,8 +135,14 @@ __device__ __forceinline__ df nblap_df(const float2* f, int m, int n, int t, int
 
 __host__ __device__ constexpr size_t coarse_df_smem(int G) { return sizeof(float2) * 7 * (size_t)G + sizeof(float) * ((size_t)G * (G + 1) + (size_t)G); }
 
-template <int SCH, int R>
-__device__ void coarse_newton_df(const DPar& P, const float* __restrict__ K3f, float2* sm) {
+__device__ __forceinline__ float df_dg32(int scheme, float p, float q) {
+  return scheme == 1 ? 3.f * p * p : 0.25f * (3.f * p * p + 2.f * p * q + q * q);
+}
+
+// One warp, a pivoted elimination in shared memory (gauss_shared) for every update: what
+// coarse_chord_df falls back to.  sm: coarse_df_smem.
+template <int SCH>
+__device__ __noinline__ void coarse_newton_df(const DPar& P, const float* __restrict__ K3f, float2* sm) {
   const DLev& C = P.L;
   const DCoef& K = P.k;
   const int m = C.m, n = C.n, G = m * n, W = G + 1;
@@ -144,7 +153,7 @@ __device__ void coarse_newton_df(const DPar& P, const float* __restrict__ K3f, f
   float2* pk = s3 + G;
   float2* pb = pk + G;
   float2* kap = pb + G;
-  float2* muv = s2;   // row 2's value replaces rho2 for an iteration (rho2 stays in global memory)
+  float2* muv = s2;   // row 2's value replaces rho2 for an iteration (rho2 stays in the level's plane)
   float* Jm = reinterpret_cast<float*>(kap + G);   // G x (G+1), last column = right-hand side
   float* d = Jm + G * W;
   const int lane = threadIdx.x & 31;
@@ -159,16 +168,7 @@ __device__ void coarse_newton_df(const DPar& P, const float* __restrict__ K3f, f
     pk[t] = (SCH == 2) ? C.pk[id] : z2;
   }
   __syncwarp();
-  constexpr int RR = R > 0 ? R : 1;
-  float k3c[RR], lcc[RR];
   const float* cLf = K3f + G * G;
-  if (R > 0) {
-#pragma unroll
-    for (int r = 0; r < RR; ++r) {
-      k3c[r] = (lane < G && r < G) ? K3f[r * G + lane] : 0.f;
-      lcc[r] = (lane < G && r < G) ? cLf[r * G + lane] : 0.f;
-    }
-  }
   auto wt = [&](int t) { return C.W ? df_of(C.W[t]) : df{0.f, 0.f}; };
   auto kappa_at = [&](int t) { return add(mk(s3[t]), mulu(mk(K.th2), nblap_df(ph, m, n, t, C.nyn))); };
   auto mu_at = [&](int t) {
@@ -177,84 +177,30 @@ __device__ void coarse_newton_df(const DPar& P, const float* __restrict__ K3f, f
     if (SCH == 2 && C.W) Q = add(Q, wt(t));
     return norm(sum3u(ldd(C.r[1] + dindex(C, t % m, t / m)), mulu(Q, dd), mulu(mk(K.ih2), nblap_df(kap, m, n, t, C.nyn))));
   };
-  auto rhs_at = [&](int t) {
-    const df f = sum3u(mk(s1[t]), neg(mk(ph[t])), mulu(mk(K.cmu), nblap_df(muv, m, n, t, C.nyn)));
-    return fadd(f.h, f.l);
-  };
-  auto diag_at = [&](int t) {   // gam + W + g'(p), the Jacobian's FP32 column factor
-    const float p = fadd(pb[t].x, ph[t].x), q = pk[t].x;
-    const float g = SCH == 1 ? 3.f * p * p : 0.25f * (3.f * p * p + 2.f * p * q + q * q);
-    return K.gam.x + (SCH == 2 && C.W ? wt(t).h : 0.f) + g;
-  };
-  bool refactor = true;
-  float dprev = 0.f;
   for (int it = 0; it < 40; ++it) {
     for (int t = lane; t < G; t += 32) kap[t] = f2(kappa_at(t));
     __syncwarp();
     for (int t = lane; t < G; t += 32) muv[t] = f2(mu_at(t));
     __syncwarp();
+    for (int t = lane; t < G; t += 32) {
+      const df f = sum3u(mk(s1[t]), neg(mk(ph[t])), mulu(mk(K.cmu), nblap_df(muv, m, n, t, C.nyn)));
+      Jm[t * W + G] = fadd(f.h, f.l);
+      d[t] = K.gam.x + (SCH == 2 && C.W ? wt(t).h : 0.f) + df_dg32(SCH, fadd(pb[t].x, ph[t].x), pk[t].x);
+    }
+    __syncwarp();
+    for (int idx = lane; idx < G * G; idx += 32) {
+      const int r = idx / G, col = idx % G;
+      Jm[r * W + col] = K3f[idx] - cLf[idx] * d[col];
+    }
+    __syncwarp();
+    gauss_shared(Jm, d, G);
     float dmax = 0.f, umax = 0.f, emax = 0.f;
-    if (R == 16) {
-      // chord iteration with J^-1 of a lagged Jacobian, as in coarse_newton
-      float* Xs = Jm;
-      float* rh = Jm + G * G;
-      int* pivs = reinterpret_cast<int*>(d);
-      for (int t = lane; t < G; t += 32) rh[t] = rhs_at(t);
-      if (refactor) {
-        for (int t = lane; t < G; t += 32) d[t] = diag_at(t);
-        __syncwarp();
-        float a[16];
-        const float dc = lane < G ? d[lane] : 0.f;
-#pragma unroll
-        for (int r = 0; r < 16; ++r)
-          a[r] = lane < G ? fmaf(-lcc[r], dc, k3c[r]) : ((lane < 2 * G && lane - G == r) ? 1.f : 0.f);
-        __syncwarp();   // d is free from here: pivot indices
-        gj_eliminate<16>(a, G, pivs);
-        if (lane >= G && lane < 2 * G)
-#pragma unroll
-          for (int r = 0; r < 16; ++r)
-            if (r < G) Xs[r * G + (lane - G)] = a[r];
-      }
-      __syncwarp();
-      float delta = 0.f;
-      if (lane < G) {
-        const float* xrow = Xs + pivs[lane] * G;
-        for (int q = 0; q < G; ++q) delta = fmaf(xrow[q], rh[q], delta);
-        const df pn = add(mk(ph[lane]), df{delta, 0.f});
-        ph[lane] = f2(pn);
-        dmax = fabsf(delta);
-        emax = fabsf(pn.h);
-        umax = fabsf(pn.h + pb[lane].x);
-      }
-    } else {
-      for (int t = lane; t < G; t += 32) Jm[t * W + G] = rhs_at(t);
-      for (int t = lane; t < G; t += 32) d[t] = diag_at(t);
-      __syncwarp();
-      if (R > 0) {
-        float a[RR];
-        const float dc = lane < G ? d[lane] : 0.f;
-#pragma unroll
-        for (int r = 0; r < RR; ++r) {
-          const float rhs = (lane == G && r < G) ? Jm[r * W + G] : 0.f;
-          a[r] = lane < G ? fmaf(-lcc[r], dc, k3c[r]) : rhs;
-        }
-        __syncwarp();   // Jm is free from here: pivot scratch
-        gauss_jordan_cols<RR>(a, G, d, Jm + G, reinterpret_cast<int*>(Jm));
-      } else {
-        for (int idx = lane; idx < G * G; idx += 32) {
-          const int r = idx / G, col = idx % G;
-          Jm[r * W + col] = K3f[idx] - cLf[idx] * d[col];
-        }
-        __syncwarp();
-        gauss_shared(Jm, d, G);
-      }
-      for (int t = lane; t < G; t += 32) {
-        const df pn = add(mk(ph[t]), df{d[t], 0.f});
-        ph[t] = f2(pn);
-        dmax = fmaxf(dmax, fabsf(d[t]));
-        emax = fmaxf(emax, fabsf(pn.h));
-        umax = fmaxf(umax, fabsf(pn.h + pb[t].x));
-      }
+    for (int t = lane; t < G; t += 32) {
+      const df pn = add(mk(ph[t]), df{d[t], 0.f});
+      ph[t] = f2(pn);
+      dmax = fmaxf(dmax, fabsf(d[t]));
+      emax = fmaxf(emax, fabsf(pn.h));
+      umax = fmaxf(umax, fabsf(pn.h + pb[t].x));
     }
     for (int o = 16; o > 0; o >>= 1) {
       dmax = fmaxf(dmax, __shfl_xor_sync(FULL, dmax, o));
@@ -263,8 +209,6 @@ __device__ void coarse_newton_df(const DPar& P, const float* __restrict__ K3f, f
     }
     __syncwarp();
     if (!(dmax == dmax) || dmax <= fmaxf(1e-15f * (1.f + umax), 1e-14f * emax)) break;
-    refactor = it > 0 && !(dmax <= 0.01f * dprev);
-    dprev = dmax;
   }
   for (int t = lane; t < G; t += 32) kap[t] = f2(kappa_at(t));
   __syncwarp();
@@ -276,12 +220,196 @@ __device__ void coarse_newton_df(const DPar& P, const float* __restrict__ K3f, f
   }
 }
 
+// Inverse of the G x G matrix entry(row, column), G <= 64, by Gauss-Jordan elimination without
+// pivoting in the registers of NT threads: thread t holds column t % 64 of rows t / 64 + NT / 64 i.
+// Before each step the owners publish the pivot row and column in shared memory (double
+// buffered: one barrier a step).  X gets the inverse column by column.  Returns false (the
+// same in every thread) where a pivot is small.
+template <int NT, typename Entry>
+__device__ __forceinline__ bool gj_invert_block(float* X, int G, Entry entry) {
+  __shared__ float prow[2][64], pcol[2][64];
+  constexpr int NG = NT / 64, NR = 64 / NG;   // NG: a power of two
+  const int q = threadIdx.x & 63, g = threadIdx.x >> 6;
+  float a[NR];
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    const int r = g + NG * i;
+    a[i] = r < G && q < G ? entry(r, q) : 0.f;
+    if (q == 0) pcol[0][r] = a[i];
+  }
+  if (g == 0) prow[0][q] = a[0];
+  __syncthreads();
+  bool ok = true;
+  for (int c = 0; c < G; ++c) {
+    const float *R = prow[c & 1], *C = pcol[c & 1];
+    const float piv = R[c], rp = __frcp_rn(piv), pq = q == c ? rp : R[q] * rp;
+    ok = ok && fabsf(piv) > 0.05f;
+    if (q < G) {
+#pragma unroll
+      for (int i = 0; i < NR; ++i)
+        if (NG * i < G) a[i] = g + NG * i == c ? pq : fmaf(-C[g + NG * i], pq, q == c ? 0.f : a[i]);
+      const int nx = c + 1;
+      if ((nx & (NG - 1)) == g)
+#pragma unroll
+        for (int i = 0; i < NR; ++i)
+          if (i == nx / NG) prow[nx & 1][q] = a[i];
+      if (q == nx)
+#pragma unroll
+        for (int i = 0; i < NR; ++i) pcol[nx & 1][g + NG * i] = a[i];
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < NR; ++i)
+    if (g + NG * i < G && q < G) X[q * G + g + NG * i] = a[i];
+  return ok;
+}
+
+// The chord iteration of warp 0 with the inverse X of a lagged Jacobian, NC cells a lane.
+// Returns false where the updates stop shrinking by 100x.
+template <int SCH, int NC>
+__device__ __forceinline__ bool coarse_chord_pass(const DPar& P, const float* X, float2* ph, float2* kap, float2* muv,
+                                                  float* rh, int& it, float& dprev) {
+  const DLev& C = P.L;
+  const DCoef& K = P.k;
+  const int m = C.m, n = C.n, G = m * n, lane = threadIdx.x;
+  int w[NC], e[NC], s[NC], u[NC], t[NC];
+  size_t id[NC];
+  df s1[NC], s2[NC], s3[NC], pb[NC], pk[NC], gw[NC], v[NC], kp[NC], mv[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    t[c] = min(lane + 32 * c, G - 1);   // a lane without a cell repeats the last one, and does not store
+    const int j = t[c] / m, i = t[c] - j * m;
+    w[c] = j * m + wrapm(i - 1, m);
+    e[c] = j * m + wrapm(i + 1, m);
+    s[c] = ywrap(j - 1, n, C.nyn) * m + i;
+    u[c] = ywrap(j + 1, n, C.nyn) * m + i;
+    id[c] = dindex(C, i, j);
+    s1[c] = ldd(C.r[0] + id[c]);
+    s2[c] = ldd(C.r[1] + id[c]);
+    s3[c] = ldd(C.r[2] + id[c]);
+    pb[c] = ldd(C.pb + id[c]);
+    pk[c] = SCH == 2 ? ldd(C.pk + id[c]) : df{0.f, 0.f};
+    gw[c] = SCH == 2 && C.W ? add(mk(K.gam), df_of(C.W[t[c]])) : mk(K.gam);
+    v[c] = ldd(ph + t[c]);
+  }
+  auto has = [&](int c) { return lane + 32 * c < G; };
+  auto lap = [&](const float2* f, int c, df own) { return lap5(ldd(f + w[c]), ldd(f + e[c]), ldd(f + s[c]), ldd(f + u[c]), own); };
+  auto rows23 = [&] {   // kappa and mu of the current d_phi
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      kp[c] = add(s3[c], mulu(mk(K.th2), lap(ph, c, v[c])));
+      if (has(c)) kap[t[c]] = f2(kp[c]);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const df Q = norm(addu(gquot<SCH>(add(pb[c], v[c]), pb[c], pk[c]), gw[c]));
+      mv[c] = norm(sum3u(s2[c], mulu(Q, v[c]), mulu(mk(K.ih2), lap(kap, c, kp[c]))));
+    }
+  };
+  bool done = false;
+#pragma unroll 1
+  for (; it < 40;) {
+    rows23();
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+      if (has(c)) muv[t[c]] = f2(mv[c]);
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const df f = sum3u(s1[c], neg(v[c]), mulu(mk(K.cmu), lap(muv, c, mv[c])));
+      if (has(c)) rh[t[c]] = fadd(f.h, f.l);
+    }
+    __syncwarp();
+    float acc[NC][2] = {};
+#pragma unroll 4
+    for (int q = 0; q < G; q += 2)   // every level has an even m
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        acc[c][0] = fmaf(X[q * G + t[c]], rh[q], acc[c][0]);
+        acc[c][1] = fmaf(X[(q + 1) * G + t[c]], rh[q + 1], acc[c][1]);
+      }
+    float dm = 0.f, em = 0.f, um = 0.f;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const float delta = acc[c][0] + acc[c][1];
+      v[c] = add(v[c], df{delta, 0.f});
+      if (has(c)) ph[t[c]] = f2(v[c]);
+      dm = fmaxf(dm, fabsf(delta));
+      if (!(delta == delta)) dm = INFINITY;
+      em = fmaxf(em, fabsf(v[c].h));
+      um = fmaxf(um, fabsf(v[c].h + pb[c].h));
+    }
+    // non-negative floats order as their bits
+    const unsigned FULL = 0xffffffffu;
+    const float dmax = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(dm)));
+    const float emax = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(em)));
+    const float umax = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(um)));
+    const float tol = fmaxf(1e-15f * (1.f + umax), 1e-14f * emax);
+    __syncwarp();
+    done = dmax <= tol || (it > 0 && dmax * (dmax / dprev) <= tol) || !(dmax < INFINITY);
+    const bool slow = it > 0 && !(dmax <= 0.01f * dprev);
+    dprev = dmax;
+    ++it;
+    if (done) break;
+    if (slow && it < 40) return false;
+  }
+  rows23();
+#pragma unroll
+  for (int c = 0; c < NC; ++c)
+    if (has(c)) {
+      C.d[0][id[c]] = f2(v[c]);
+      C.d[1][id[c]] = f2(mv[c]);
+      C.d[2][id[c]] = f2(kp[c]);
+    }
+  return true;
+}
+
+// The coarsest solve of a CTA of kDfTailThreads threads: J^-1 of the Jacobian at d = 0 by all of them
+// (gj_invert_block), updates J^-1 F by warp 0, J^-1 again where they shrink slowly; the
+// pivoting solve where a pivot is small (|.| <= 0.05: J = I + (-c L)(diag(q) + theta L^2) has a
+// positive diagonal unless q < 0 dominates) or four inverses were not enough.  sm: coarse_df_smem.
+// Bound by the serial chain of the eliminations' steps and of the updates: an elimination by one
+// warp for every update on 8 x 6 cells, the coarse tail of 512 x 384, made that kernel 151 us, now
+// 71; on 4 x 4 cells (1024^2) a warp's Gauss-Jordan elimination 40.3, now 38.7.
 template <int SCH>
-__device__ void coarse_df_warp(const DPar& P, const float* __restrict__ K3f, float2* sm) {
-  const int G = P.L.m * P.L.n;
-  if (G <= 16) coarse_newton_df<SCH, 16>(P, K3f, sm);
-  else if (G <= 31) coarse_newton_df<SCH, 32>(P, K3f, sm);
-  else coarse_newton_df<SCH, 0>(P, K3f, sm);
+__device__ __forceinline__ void coarse_df_block(const DPar& P, const float* __restrict__ K3f, float2* sm) {
+  __shared__ int s_state;   // 0: solved, 1: a new inverse
+  const DLev& C = P.L;
+  const int G = C.m * C.n;
+  float2* ph = sm;
+  float2* kap = ph + G;
+  float2* muv = kap + G;
+  float* diag = reinterpret_cast<float*>(muv + G);
+  float* rh = diag + G;
+  float* X = rh + G;
+  const float* cLf = K3f + G * G;
+  const int tid = threadIdx.x;
+  if (tid < G) ph[tid] = make_float2(0.f, 0.f);
+  int it = 0;
+  float dprev = 0.f;
+  for (int f = 0;; ++f) {
+    if (tid < G) {   // gam + W + g'(p), the Jacobian's FP32 column factor
+      const size_t id = dindex(C, tid % C.m, tid / C.m);
+      diag[tid] = P.k.gam.x + (SCH == 2 && C.W ? df_of(C.W[tid]).h : 0.f) +
+                  df_dg32(SCH, fadd(C.pb[id].x, ph[tid].x), SCH == 2 ? C.pk[id].x : 0.f);
+    }
+    __syncthreads();
+    if (f == 4 || !gj_invert_block<kDfTailThreads>(X, G, [&](int r, int q) { return fmaf(-cLf[r * G + q], diag[q], K3f[r * G + q]); })) {
+      __syncthreads();
+      if (tid < 32) coarse_newton_df<SCH>(P, K3f, sm);
+      return;
+    }
+    __syncthreads();
+    if (tid < 32) {
+      const bool ok = G <= 32 ? coarse_chord_pass<SCH, 1>(P, X, ph, kap, muv, rh, it, dprev)
+                              : coarse_chord_pass<SCH, 2>(P, X, ph, kap, muv, rh, it, dprev);
+      if (tid == 0) s_state = ok ? 0 : 1;
+    }
+    __syncthreads();
+    if (s_state == 0) return;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -291,8 +419,6 @@ __device__ void coarse_df_warp(const DPar& P, const float* __restrict__ K3f, flo
 // and its correction is written back at the end; coarser levels exist in shared memory only
 // (their phi^k excepted).  Levels that do not fit stay in global memory.
 // ---------------------------------------------------------------------------
-constexpr int kDfTailMax = 10;
-constexpr int kDfTailThreads = 512;
 constexpr size_t kDfTailSmem = 160 * 1024;
 
 struct DTailDim {
@@ -370,7 +496,7 @@ __device__ __forceinline__ void df_tail_body(const DTailDim& A, const DPar* lv, 
     for (int t = tid; t < cc; t += nt) df_restrict_cell<SCH, true, true>(F, C, t % C.L.m, t / C.L.m, zero);
     __syncthreads();
   }
-  if (tid < 32) coarse_df_warp<SCH>(sl[A.nlev - 1], k3s, scratch);
+  coarse_df_block<SCH>(sl[A.nlev - 1], k3s, scratch);
   __syncthreads();
   for (int l = A.nlev - 2; l >= 0; --l) {
     const DPar& F = sl[l];

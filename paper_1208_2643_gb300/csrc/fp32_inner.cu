@@ -59,7 +59,7 @@ dim3 grid_of(int X, int Y) { return dim3((X + kBlk.x - 1) / kBlk.x, (Y + kBlk.y 
 // e = 0, and the scaled residual norm with the outer loop decision.  Bound by the FP64 pipe
 // (8 instructions a cell in scheme 1, the Laplacians being integer sums, lap5_f64); the
 // linearisation and, after the first cycle, the squares are float-float (as in
-// df_defect_cell): @D@ us at 1024^2, 75 with all of it in FP64.
+// df_defect_pair): 40 us at 1024^2, 75 with all of it in FP64.
 // ---------------------------------------------------------------------------
 template <int SCH>
 __global__ void __launch_bounds__(256, 5) k_defect(Lev L, Coef k, Lev32 E, Ctl* ctl, double* partials, int mode,
