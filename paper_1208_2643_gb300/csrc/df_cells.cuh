@@ -98,7 +98,7 @@ __device__ __forceinline__ void df_update(const DCoef& K, df Lp, df Lm, df Lk, D
     r1 = add(c.rho1, mulu(mk(K.cmu), Lm));
     r2 = add(c.rho2, mulu(mk(K.ih2), Lk));
     r3 = add(c.rho3, mulu(mk(K.th2), Lp));
-    p = c.pb;
+    p = norm(c.pb);   // with this, the bits of kGen on a zero correction
   } else {
     p = add(c.pb, c.p);
     r1 = norm(sum3u(c.rho1, mulu(mk(K.cmu), Lm), neg(c.p)));

@@ -18,7 +18,7 @@ using namespace mpfc;
 namespace {
 
 // ---------------------------------------------------------------------------
-// FP64 residual of the iterate (df_defect_cell), the scaled norm and the loop decision.
+// FP64 residual of the iterate (df_defect_pair), the scaled norm and the loop decision.
 // A value outside the range the float-float form covers (|phi| < 2^20, |rho| < 2^40: far
 // inside binary32, the cubic included) sets ctl->range; the loop then goes on with the
 // FP64 V-cycle.

@@ -220,44 +220,68 @@ __device__ __noinline__ void coarse_newton_df(const DPar& P, const float* __rest
   }
 }
 
-// Inverse of the G x G matrix entry(row, column), G <= 64, by Gauss-Jordan elimination without
-// pivoting in the registers of NT threads: thread t holds column t % 64 of rows t / 64 + NT / 64 i.
-// Before each step the owners publish the pivot row and column in shared memory (double
-// buffered: one barrier a step).  X gets the inverse column by column.  Returns false (the
-// same in every thread) where a pivot is small.
-template <int NT, typename Entry>
+// Inverse of the G x G matrix entry(row, column) by Gauss-Jordan elimination without pivoting in
+// the registers of a CTA of NT threads: CW columns (CW >= G), thread t holds column t % CW of rows
+// t / CW + NG i.  Before each step the owners publish the pivot row and column in shared
+// memory, double buffered: one barrier a step, of the threads that hold rows.  The elimination
+// is a chain of G steps, so a step's instructions count: the column's entries are read four at
+// a time, and a thread of the pivot column needs no select (its entry is the published one,
+// C - C (1 + 1/piv) = -C / piv).  X gets the inverse column by column.  Returns false (the same
+// in every thread that holds rows) where a pivot is small.
+template <int NT, int CW, typename Entry>
 __device__ __forceinline__ bool gj_invert_block(float* X, int G, Entry entry) {
-  __shared__ float prow[2][64], pcol[2][64];
-  constexpr int NG = NT / 64, NR = 64 / NG;   // NG: a power of two
-  const int q = threadIdx.x & 63, g = threadIdx.x >> 6;
+  constexpr int NG = NT / CW < CW ? NT / CW : CW, NR = CW / NG;   // powers of two
+  __shared__ __align__(16) float prow[2][CW], pcol[2][CW];        // pcol: row g + NG i at NR g + i
+  const int q = threadIdx.x % CW, g = threadIdx.x / CW;
+  if (g >= NG) return true;
+  auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(NG * CW) : "memory"); };
   float a[NR];
 #pragma unroll
   for (int i = 0; i < NR; ++i) {
     const int r = g + NG * i;
     a[i] = r < G && q < G ? entry(r, q) : 0.f;
-    if (q == 0) pcol[0][r] = a[i];
+    if (q == 0) pcol[0][NR * g + i] = a[i];
   }
   if (g == 0) prow[0][q] = a[0];
-  __syncthreads();
+  sync();
   bool ok = true;
   for (int c = 0; c < G; ++c) {
-    const float *R = prow[c & 1], *C = pcol[c & 1];
-    const float piv = R[c], rp = __frcp_rn(piv), pq = q == c ? rp : R[q] * rp;
-    ok = ok && fabsf(piv) > 0.05f;
-    if (q < G) {
+    const float* R = prow[c & 1];
+    const float* C = pcol[c & 1] + NR * g;
+    const float piv = R[c], rq = R[q];
+    float f[NR];
+    if (NR >= 4) {
 #pragma unroll
-      for (int i = 0; i < NR; ++i)
-        if (NG * i < G) a[i] = g + NG * i == c ? pq : fmaf(-C[g + NG * i], pq, q == c ? 0.f : a[i]);
-      const int nx = c + 1;
-      if ((nx & (NG - 1)) == g)
+      for (int i = 0; i < NR; i += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(C + i);
+        f[i] = v.x; f[i + 1] = v.y; f[i + 2] = v.z; f[i + 3] = v.w;
+      }
+    } else {
 #pragma unroll
-        for (int i = 0; i < NR; ++i)
-          if (i == nx / NG) prow[nx & 1][q] = a[i];
-      if (q == nx)
-#pragma unroll
-        for (int i = 0; i < NR; ++i) pcol[nx & 1][g + NG * i] = a[i];
+      for (int i = 0; i < NR; ++i) f[i] = C[i];
     }
-    __syncthreads();
+    float rp;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rp) : "f"(piv));
+    ok = ok && fabsf(piv) > 0.05f;
+    const float pq = q == c ? 1.f + rp : rq * rp;
+#pragma unroll
+    for (int i = 0; i < NR; ++i) a[i] = fmaf(-f[i], pq, a[i]);
+    if (c % NG == g) {
+      const float v = q == c ? rp : pq;
+#pragma unroll
+      for (int i = 0; i < NR; ++i) a[i] = i == c / NG ? v : a[i];
+    }
+    const int nx = c + 1;
+    if (nx % NG == g) {
+      float v = a[0];
+#pragma unroll
+      for (int i = 1; i < NR; ++i) v = i == nx / NG ? a[i] : v;
+      prow[nx & 1][q] = v;
+    }
+    if (q == nx)
+#pragma unroll
+      for (int i = 0; i < NR; ++i) pcol[nx & 1][NR * g + i] = a[i];
+    sync();
   }
 #pragma unroll
   for (int i = 0; i < NR; ++i)
@@ -396,16 +420,23 @@ __device__ __forceinline__ void coarse_df_block(const DPar& P, const float* __re
                   df_dg32(SCH, fadd(C.pb[id].x, ph[tid].x), SCH == 2 ? C.pk[id].x : 0.f);
     }
     __syncthreads();
-    if (f == 4 || !gj_invert_block<kDfTailThreads>(X, G, [&](int r, int q) { return fmaf(-cLf[r * G + q], diag[q], K3f[r * G + q]); })) {
-      __syncthreads();
-      if (tid < 32) coarse_newton_df<SCH>(P, K3f, sm);
-      return;
+    auto entry = [&](int r, int q) { return fmaf(-cLf[r * G + q], diag[q], K3f[r * G + q]); };
+    bool ok = f < 4;
+    if (ok) {
+      if (G <= 16) ok = gj_invert_block<kDfTailThreads, 16>(X, G, entry);
+      else if (G <= 32) ok = gj_invert_block<kDfTailThreads, 32>(X, G, entry);
+      else ok = gj_invert_block<kDfTailThreads, 64>(X, G, entry);
     }
     __syncthreads();
-    if (tid < 32) {
-      const bool ok = G <= 32 ? coarse_chord_pass<SCH, 1>(P, X, ph, kap, muv, rh, it, dprev)
-                              : coarse_chord_pass<SCH, 2>(P, X, ph, kap, muv, rh, it, dprev);
-      if (tid == 0) s_state = ok ? 0 : 1;
+    if (tid < 32) {   // warp 0 holds rows: its ok is every such thread's
+      if (!ok) {
+        coarse_newton_df<SCH>(P, K3f, sm);
+        if (tid == 0) s_state = 0;
+      } else {
+        const bool done = G <= 32 ? coarse_chord_pass<SCH, 1>(P, X, ph, kap, muv, rh, it, dprev)
+                                  : coarse_chord_pass<SCH, 2>(P, X, ph, kap, muv, rh, it, dprev);
+        if (tid == 0) s_state = done ? 0 : 1;
+      }
     }
     __syncthreads();
     if (s_state == 0) return;
@@ -424,16 +455,6 @@ constexpr size_t kDfTailSmem = 160 * 1024;
 struct DTailDim {
   int nlev, nu1, nu2, staged;   // levels 0 .. staged-1 of the tail stay in global memory
 };
-
-template <int SCH, int MODE, bool NY>
-__device__ __forceinline__ void df_tail_half(const DPar& P, int color) {
-  const int half = P.L.m >> 1, cells = half * P.L.n;
-  for (int t = threadIdx.x; t < cells; t += blockDim.x) {
-    const int j = t / half;
-    df_smooth_cell<SCH, MODE, NY, false>(P, color, t - j * half, j);
-  }
-  __syncthreads();
-}
 
 // lv: the levels' parameters; ready(): called once before any data another kernel wrote is read.
 template <int SCH, bool NY, typename Ready>
@@ -468,7 +489,20 @@ __device__ __forceinline__ void df_tail_body(const DTailDim& A, const DPar* lv, 
     }
   }
   __syncthreads();
+  // the black half of d is zero before a level's first sweep (whose red half sweep the
+  // restriction did): in global memory after the wait, in shared memory before it
+  auto zero_black = [&](int l) {
+    const DLev& v = sl[l].L;
+    const int h = (v.m >> 1) * v.n;
+    for (int t = tid; t < h; t += nt)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) v.d[c][h + t] = make_float2(0.f, 0.f);
+  };
+  for (int l = A.staged; l < A.nlev; ++l) zero_black(l);
   ready();
+  if (A.nu1 > 0)
+    for (int l = 0; l < A.staged; ++l) zero_black(l);
+  __syncthreads();
   if (A.staged == 0) {   // the tail's first level comes in from global memory
     const DLev& g = lv[0].L;
     const DLev& v = sl[0].L;
@@ -483,32 +517,38 @@ __device__ __forceinline__ void df_tail_body(const DTailDim& A, const DPar* lv, 
     }
     __syncthreads();
   }
-  for (int l = 0; l < A.nlev - 1; ++l) {
+  // down and up as one loop, with one copy of the sweep's code: what a copy costs on its first
+  // use (2 to 10 k clocks of instruction fetch) is several warm half sweeps (1.3 k)
+  const int down = A.nlev - 1;
+  for (int leg = 0; leg < 2 * down; ++leg) {
+    const bool up = leg >= down;
+    const int l = up ? 2 * down - 1 - leg : leg;
     const DPar& F = sl[l];
     const DPar& C = sl[l + 1];
-    if (A.nu1 > 0) {
-      df_tail_half<SCH, kOwn, NY>(F, 1);
-      for (int sw = 1; sw < A.nu1; ++sw)
-        for (int color = 0; color < 2; ++color) df_tail_half<SCH, kGen, NY>(F, color);
+    const int half = F.L.m >> 1, cells = half * F.L.n, cc = C.L.m * C.L.n;
+    if (up) {
+      for (int t = tid; t < 3 * cc; t += nt) {
+        const int c = t / cc, q = t - c * cc;
+        df_prolong_plane(C.L, F.L, c, q % C.L.m, q / C.L.m);
+      }
+      __syncthreads();
     }
-    const int cc = C.L.m * C.L.n;
-    const int zero = A.nu1 == 0 || l + 1 == A.nlev - 1;
-    for (int t = tid; t < cc; t += nt) df_restrict_cell<SCH, true, true>(F, C, t % C.L.m, t / C.L.m, zero);
-    __syncthreads();
-  }
-  coarse_df_block<SCH>(sl[A.nlev - 1], k3s, scratch);
-  __syncthreads();
-  for (int l = A.nlev - 2; l >= 0; --l) {
-    const DPar& F = sl[l];
-    const DPar& C = sl[l + 1];
-    const int cc = C.L.m * C.L.n;
-    for (int t = tid; t < 3 * cc; t += nt) {
-      const int c = t / cc, q = t - c * cc;
-      df_prolong_plane(C.L, F.L, c, q % C.L.m, q / C.L.m);
+    for (int hs = up ? 0 : 1; hs < 2 * (up ? A.nu2 : A.nu1); ++hs) {
+      for (int t = tid; t < cells; t += nt) {
+        const int j = t / half;
+        df_smooth_cell<SCH, kGen, NY, false>(F, hs & 1, t - j * half, j);
+      }
+      __syncthreads();
     }
-    __syncthreads();
-    for (int sw = 0; sw < A.nu2; ++sw)
-      for (int color = 0; color < 2; ++color) df_tail_half<SCH, kGen, NY>(F, color);
+    if (!up) {
+      const int zero = A.nu1 == 0 || l + 1 == down;
+      for (int t = tid; t < cc; t += nt) df_restrict_cell<SCH, true, true>(F, C, t % C.L.m, t / C.L.m, zero);
+      __syncthreads();
+      if (l + 1 == down) {
+        coarse_df_block<SCH>(sl[down], k3s, scratch);
+        __syncthreads();
+      }
+    }
   }
   if (A.staged == 0) {
     const DLev& g = lv[0].L;
