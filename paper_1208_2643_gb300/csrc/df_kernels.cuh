@@ -231,7 +231,7 @@ __device__ __noinline__ void coarse_newton_df(const DPar& P, const float* __rest
 template <int NT, int CW, typename Entry>
 __device__ __forceinline__ bool gj_invert_block(float* X, int G, Entry entry) {
   constexpr int NG = NT / CW < CW ? NT / CW : CW, NR = CW / NG;   // powers of two
-  __shared__ __align__(16) float prow[2][CW], pcol[2][CW];        // pcol: row g + NG i at NR g + i
+  __shared__ __align__(16) float prow[2][CW], pcol[2][CW];        // pcol: a[i] of group g at NR g + i
   const int q = threadIdx.x % CW, g = threadIdx.x / CW;
   if (g >= NG) return true;
   auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(NG * CW) : "memory"); };
@@ -266,26 +266,25 @@ __device__ __forceinline__ bool gj_invert_block(float* X, int G, Entry entry) {
     const float pq = q == c ? 1.f + rp : rq * rp;
 #pragma unroll
     for (int i = 0; i < NR; ++i) a[i] = fmaf(-f[i], pq, a[i]);
-    if (c % NG == g) {
-      const float v = q == c ? rp : pq;
-#pragma unroll
-      for (int i = 0; i < NR; ++i) a[i] = i == c / NG ? v : a[i];
-    }
+    if ((c & (NG - 1)) == g) a[0] = q == c ? rp : pq;
     const int nx = c + 1;
-    if (nx % NG == g) {
-      float v = a[0];
+    if ((nx & (NG - 1)) == 0) {   // the next rows' register comes first (a register array has no index)
+      const float t = a[0];
 #pragma unroll
-      for (int i = 1; i < NR; ++i) v = i == nx / NG ? a[i] : v;
-      prow[nx & 1][q] = v;
+      for (int i = 1; i < NR; ++i) a[i - 1] = a[i];
+      a[NR - 1] = t;
     }
+    if ((nx & (NG - 1)) == g) prow[nx & 1][q] = a[0];
     if (q == nx)
 #pragma unroll
       for (int i = 0; i < NR; ++i) pcol[nx & 1][NR * g + i] = a[i];
     sync();
   }
 #pragma unroll
-  for (int i = 0; i < NR; ++i)
-    if (g + NG * i < G && q < G) X[q * G + g + NG * i] = a[i];
+  for (int i = 0; i < NR; ++i) {
+    const int r = g + NG * ((i + G / NG) & (NR - 1));
+    if (r < G && q < G) X[q * G + r] = a[i];
+  }
   return ok;
 }
 
@@ -396,7 +395,8 @@ __device__ __forceinline__ bool coarse_chord_pass(const DPar& P, const float* X,
 // positive diagonal unless q < 0 dominates) or four inverses were not enough.  sm: coarse_df_smem.
 // Bound by the serial chain of the eliminations' steps and of the updates: an elimination by one
 // warp for every update on 8 x 6 cells, the coarse tail of 512 x 384, made that kernel 151 us, now
-// 71; on 4 x 4 cells (1024^2) a warp's Gauss-Jordan elimination 40.3, now 38.7.
+// 44; on 4 x 4 cells (1024^2) a warp's Gauss-Jordan elimination and a tail of three copies of the
+// sweep's code 40, now 28.
 template <int SCH>
 __device__ __forceinline__ void coarse_df_block(const DPar& P, const float* __restrict__ K3f, float2* sm) {
   __shared__ int s_state;   // 0: solved, 1: a new inverse
