@@ -317,8 +317,10 @@ __global__ void __launch_bounds__(kTX * kTY) k_prolong32(Lev32 F, Lev32 C) {
 // ---------------------------------------------------------------------------
 // Coarsest grid, FP32: eliminate e_kappa and e_mu,
 //   (I - c L diag(q) - c theta L^3) e_phi = r1 + c L (r2 + L r3),
-// solve by Gaussian elimination with partial pivoting in one CTA, then
-// e_kappa = r3 + theta L e_phi, e_mu = r2 + q e_phi + L e_kappa.
+// solve in one CTA, then e_kappa = r3 + theta L e_phi, e_mu = r2 + q e_phi + L e_kappa.
+// The solve is an inverse (gj_invert_block, a barrier a step) and one refinement of its
+// solution; Gaussian elimination with partial pivoting, several barriers and a one-thread
+// search a column, where a pivot is small.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float nbsum32(const float* f, int m, int n, int t, int nyn) {
   int i = t % m, j = t / m;
@@ -326,8 +328,9 @@ __device__ __forceinline__ float nbsum32(const float* f, int m, int n, int t, in
          (f[ywrap(j - 1, n, nyn) * m + i] + f[ywrap(j + 1, n, nyn) * m + i]);
 }
 
-// The whole block; smf holds G (G + 1) + 4 G floats.  C's planes may be in global or
+// All threads of a CTA of kTail32Threads; smf holds G (G + 1) + 4 G floats.  C's planes may be in global or
 // shared memory (plain loads).
+constexpr int kTail32Threads = 1024;
 __device__ void coarse32_block(const Lev32& C, const Coef32& k, const float* __restrict__ K3f, float* smf) {
   const int m = C.m, n = C.n, G = m * n, W = G + 1;
   float* A = smf;
@@ -342,32 +345,35 @@ __device__ void coarse32_block(const Lev32& C, const Coef32& k, const float* __r
   __syncthreads();
   for (int t = tid; t < G; t += nt) t2[t] = C.r2[t] + t1[t];
   __syncthreads();
-  for (int t = tid; t < G; t += nt) A[t * W + G] = C.r1[t] + k.cmu * (nbsum32(t2, m, n, t, C.nyn) - 4.f * t2[t]);
+  for (int t = tid; t < G; t += nt) d[t] = C.r1[t] + k.cmu * (nbsum32(t2, m, n, t, C.nyn) - 4.f * t2[t]);
   const float* cLf = K3f + G * G;   // c L, after K3 in the coarse block
   auto entry = [&](int r, int col) { return K3f[r * G + col] - cLf[r * G + col] * C.q[col]; };
-  if (G <= 31) {
-    // one warp: a Jacobian column per lane in registers, Gauss-Jordan with implicit
-    // pivoting (gauss_jordan_cols); the right-hand side in lane G
-    __syncthreads();
-    auto column = [&](auto& a) {
-      constexpr int R = sizeof(a) / sizeof(a[0]);
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-        a[r] = (r < G) ? (tid < G ? entry(r, tid) : (tid == G ? A[r * W + G] : 0.f)) : 0.f;
-      __syncwarp();
-      gauss_jordan_cols<R>(a, G, x, t2, reinterpret_cast<int*>(d));
-    };
-    if (tid < 32) {
-      if (G <= 16) {
-        float a[16];
-        column(a);
-      } else {
-        float a[32];
-        column(a);
+  bool ok;
+  if (G <= 16) ok = gj_invert_block<kTail32Threads, 16>(A, G, entry);
+  else if (G <= 32) ok = gj_invert_block<kTail32Threads, 32>(A, G, entry);
+  else ok = gj_invert_block<kTail32Threads, 64>(A, G, entry);
+  if (__syncthreads_and(ok)) {
+    auto apply = [&](const float* b, float acc) {   // row tid of A^-1 b
+      float a1 = 0.f;
+      for (int q = 0; q < G; q += 2) {   // every level has an even m
+        acc = fmaf(A[q * G + tid], b[q], acc);
+        a1 = fmaf(A[(q + 1) * G + tid], b[q + 1], a1);
       }
+      return acc + a1;
+    };
+    if (tid < G) x[tid] = apply(d, 0.f);
+    __syncthreads();
+    if (tid < G) {
+      float r = d[tid];
+      for (int q = 0; q < G; ++q) r = fmaf(-entry(tid, q), x[q], r);
+      t1[tid] = r;
     }
     __syncthreads();
+    if (tid < G) x[tid] = apply(t1, x[tid]);
+    __syncthreads();
   } else {
+    for (int t = tid; t < G; t += nt) A[t * W + G] = d[t];
+    __syncthreads();
     for (int idx = tid; idx < G * G; idx += nt) A[(idx / G) * W + idx % G] = entry(idx / G, idx % G);
     __syncthreads();
     for (int col = 0; col < G; ++col) {
@@ -415,7 +421,7 @@ __device__ void coarse32_block(const Lev32& C, const Coef32& k, const float* __r
   }
 }
 
-__global__ void k_coarse32(Lev32 C, Coef32 k, const float* __restrict__ K3f) {
+__global__ void __launch_bounds__(kTail32Threads) k_coarse32(Lev32 C, Coef32 k, const float* __restrict__ K3f) {
   pdl_enter();
   extern __shared__ float smf[];
   coarse32_block(C, k, K3f, smf);
@@ -881,10 +887,10 @@ int inner_cycles_of(const mpfc_s* H) { return H->p.inner_cycles > 0 ? H->p.inner
 // (so the same bits), separated by __syncthreads instead of kernel boundaries.  The
 // FP32 work of a small level is far below a launch's cost.  Level lt's correction is
 // read at the start and written back at the end; its defect source and every level's
-// q are read from the global planes.
+// q are read from the global planes.  Bound by the chain of its phases: 29 us from 16^2 to 4^2
+// (45 with a one-warp elimination and a second copy of the code for the way up).
 // ---------------------------------------------------------------------------
 constexpr int kMaxTail32 = 8;
-constexpr int kTail32Threads = 1024;
 constexpr size_t kTail32MaxSmem = 200 * 1024;   // dynamic shared memory, below the 227 KB opt-in limit
 
 struct Tail32Args {
@@ -960,44 +966,39 @@ __global__ void __launch_bounds__(kTail32Threads) k_tail32(const __grid_constant
     }
   }
   __syncthreads();
-  for (int l = 0; l < A.nlev - 1; ++l) {
+  // down and up as one loop, with one copy of the sweep's code (a copy's first use costs more
+  // in instruction fetch than a warm half sweep)
+  const int down = A.nlev - 1;
+  for (int leg = 0; leg < 2 * down; ++leg) {
+    const bool up = leg >= down;
+    const int l = up ? 2 * down - 1 - leg : leg;
     const Lev32& F = sl[l];
     const Lev32& C = sl[l + 1];
-    const int half = F.m >> 1, hc = half * F.n;
-    for (int sw = 0; sw < A.nu1; ++sw)
-      for (int color = 0; color < 2; ++color) {
-        for (int t = tid; t < hc; t += nt) {
-          const int j = t / half, x = t - j * half;
-          smooth32_cell<false>(F, A.k[l], A.kb[l], 2 * x + ((j + color) & 1), j);
-        }
-        __syncthreads();
+    const int half = F.m >> 1, hc = half * F.n, fc = F.m * F.n, cc = C.m * C.n;
+    if (up) {
+      for (int t = tid; t < fc; t += nt) {
+        const int fi = t % F.m, fj = t / F.m;
+        prolong32_fine(C.ephi, F.ephi, C.m, C.n, C.nyn, fi, fj);
+        prolong32_fine(C.emu, F.emu, C.m, C.n, C.nyn, fi, fj);
+        prolong32_fine(C.eka, F.eka, C.m, C.n, C.nyn, fi, fj);
       }
-    const int cc = C.m * C.n;
-    for (int t = tid; t < cc; t += nt) restrict_defect32_cell<false>(F, C, A.k[l], t % C.m, t / C.m);
-    __syncthreads();
-  }
-  coarse32_block(sl[A.nlev - 1], A.k[A.nlev - 1], k3s, scratch);
-  __syncthreads();
-  for (int l = A.nlev - 2; l >= 0; --l) {
-    const Lev32& F = sl[l];
-    const Lev32& C = sl[l + 1];
-    const int fc = F.m * F.n;
-    for (int t = tid; t < fc; t += nt) {
-      const int fi = t % F.m, fj = t / F.m;
-      prolong32_fine(C.ephi, F.ephi, C.m, C.n, C.nyn, fi, fj);
-      prolong32_fine(C.emu, F.emu, C.m, C.n, C.nyn, fi, fj);
-      prolong32_fine(C.eka, F.eka, C.m, C.n, C.nyn, fi, fj);
+      __syncthreads();
     }
-    __syncthreads();
-    const int half = F.m >> 1, hc = half * F.n;
-    for (int sw = 0; sw < A.nu2; ++sw)
-      for (int color = 0; color < 2; ++color) {
-        for (int t = tid; t < hc; t += nt) {
-          const int j = t / half, x = t - j * half;
-          smooth32_cell<false>(F, A.k[l], A.kb[l], 2 * x + ((j + color) & 1), j);
-        }
+    for (int hs = 0; hs < 2 * (up ? A.nu2 : A.nu1); ++hs) {
+      for (int t = tid; t < hc; t += nt) {
+        const int j = t / half, x = t - j * half;
+        smooth32_cell<false>(F, A.k[l], A.kb[l], 2 * x + ((j + hs) & 1), j);
+      }
+      __syncthreads();
+    }
+    if (!up) {
+      for (int t = tid; t < cc; t += nt) restrict_defect32_cell<false>(F, C, A.k[l], t % C.m, t / C.m);
+      __syncthreads();
+      if (l + 1 == down) {
+        coarse32_block(sl[down], A.k[down], k3s, scratch);
         __syncthreads();
       }
+    }
   }
   {
     const Lev32& T = sl[0];
@@ -1056,7 +1057,7 @@ void enqueue_inner_vcycle(mpfc_s* H, int scheme, cudaStream_t s) {
     launch_tail32(H, scheme, lt, s);
   } else {
     const Lev32& Cc = H->lev32[L - 1];
-    mpfc_launch(sh, k_coarse32, dim3(1), dim3(256), coarse32_smem(Cc), s, Cc, coef32_of(H->coef[scheme - 1][L - 1]),
+    mpfc_launch(sh, k_coarse32, dim3(1), dim3(kTail32Threads), coarse32_smem(Cc), s, Cc, coef32_of(H->coef[scheme - 1][L - 1]),
                 (const float*)H->K3f[scheme - 1]);
   }
   for (int l = down - 1; l >= 0; --l) {
