@@ -258,9 +258,10 @@ __device__ __forceinline__ df mul2(df a, float k) { return scale2(a, k); }
 // Restriction at coarse cell (I, J): rho_c = R r and p0_c = R(p0 + d_phi).  The block sum of
 // the five-point Laplacian is (sum of the 8 bordering cells - 2 sum of the block) / h^2, as in
 // the FP64 form.  FIRST: also the first red half sweep of the coarse level (d_c = 0 before
-// it), on the values in registers; BASE: p0_c here (else by df_base_cell).
+// it), on the values in registers; BASE: p0_c here (else by df_base_cell).  (cI, cJ): the
+// coarse cell in PC, where PF is a staged part of the fine level and (I, J) counts from its origin.
 template <int SCH, bool FIRST, bool BASE>
-__device__ __forceinline__ void df_restrict_cell(const DPar& PF, const DPar& PC, int I, int J, int zero) {
+__device__ __forceinline__ void df_restrict_cell(const DPar& PF, const DPar& PC, int I, int J, int zero, int cI, int cJ) {
   const DLev& F = PF.L;
   const DLev& C = PC.L;
   const DCoef& K = PF.k;
@@ -283,7 +284,7 @@ __device__ __forceinline__ void df_restrict_cell(const DPar& PF, const DPar& PC,
   const df c1 = scale2(norm(sum3u(rho1, mulu(mk(K.cmu), lm), neg(sp))), 0.25f);
   const df c2 = scale2(norm(sum4u(rho2, mulu(mk(K.ih2), lk), neg(sm), gs)), 0.25f);
   const df c3 = scale2(norm(sum3u(rho3, mulu(mk(K.th2), lp), neg(sk))), 0.25f);
-  const size_t cid = dindex(C, I, J);
+  const size_t cid = dindex(C, cI, cJ);
   C.r[0][cid] = f2(c1);
   C.r[1][cid] = f2(c2);
   C.r[2][cid] = f2(c3);
@@ -294,7 +295,7 @@ __device__ __forceinline__ void df_restrict_cell(const DPar& PF, const DPar& PC,
     C.d[0][cid] = z;
     C.d[1][cid] = z;
     C.d[2][cid] = z;
-  } else if (FIRST && !((I + J) & 1)) {
+  } else if (FIRST && !((cI + cJ) & 1)) {
     DCell c;
     c.rho1 = c1;
     c.rho2 = c2;
@@ -302,14 +303,19 @@ __device__ __forceinline__ void df_restrict_cell(const DPar& PF, const DPar& PC,
     c.pb = pbc;
     c.pk = (SCH == 2) ? ldd(C.pk + cid) : df{0.f, 0.f};
     c.W = df{0.f, 0.f};
-    if (SCH == 2 && C.W) c.W = df_of(C.W[(size_t)J * C.m + I]);
+    if (SCH == 2 && C.W) c.W = df_of(C.W[(size_t)cJ * C.m + cI]);
     const df z{0.f, 0.f};
-    if (C.nyn && (J == 0 || J == C.n - 1)) df_update<SCH, kAll>(PC.kb, z, z, z, c);
+    if (C.nyn && (cJ == 0 || cJ == C.n - 1)) df_update<SCH, kAll>(PC.kb, z, z, z, c);
     else df_update<SCH, kAll>(PC.k, z, z, z, c);
     C.d[0][cid] = f2(c.p);
     C.d[1][cid] = f2(c.m);
     C.d[2][cid] = f2(c.k);
   }
+}
+
+template <int SCH, bool FIRST, bool BASE>
+__device__ __forceinline__ void df_restrict_cell(const DPar& PF, const DPar& PC, int I, int J, int zero) {
+  df_restrict_cell<SCH, FIRST, BASE>(PF, PC, I, J, zero, I, J);
 }
 
 // p0_c = R(p0 + d_phi) alone, with the operations of df_restrict_cell.
@@ -322,8 +328,17 @@ __device__ __forceinline__ void df_base_cell(const DLev& F, const DLev& C, int I
   C.pb[dindex(C, I, J)] = f2(scale2(add(sb, sp), 0.25f));
 }
 
-// Prolongation into the four children of coarse cell (I, J): d_f += P d_c, weights
-// (9, 3, 3, 1)/16 (9 e = 8 e + e and 3 e = 2 e + e, both with exact power-of-two terms).
+// The prolonged correction at a fine cell: weights (9, 3, 3, 1)/16 of the coarse cell that holds
+// it, its neighbours in x and y on the fine cell's side, and the diagonal one (9 e = 8 e + e and
+// 3 e = 2 e + e, both with exact power-of-two terms).  c9 = 9/16 e.
+__device__ __forceinline__ df df_nine(df e) { return add(scale2(e, 0.5f), scale2(e, 0.0625f)); }
+__device__ __forceinline__ df df_bilinear(df c9, df x, df y, df xy) {
+  const df s = add(x, y);
+  return norm(sum4u(c9, scale2(s, 0.125f), scale2(s, 0.0625f), scale2(xy, 0.0625f)));
+}
+__device__ __forceinline__ df df_prolonged(df e, df x, df y, df xy) { return df_bilinear(df_nine(e), x, y, xy); }
+
+// Prolongation into the four children of coarse cell (I, J): d_f += P d_c.
 __device__ __forceinline__ void df_prolong_plane(const DLev& C, const DLev& F, int c, int I, int J) {
   const float2* e = C.d[c];
   const int Iw = I > 0 ? I - 1 : C.m - 1, Ie = I < C.m - 1 ? I + 1 : 0;
@@ -331,7 +346,7 @@ __device__ __forceinline__ void df_prolong_plane(const DLev& C, const DLev& F, i
   const df e00 = ldd(e + dindex(C, I, J));
   const df eW = ldd(e + dindex(C, Iw, J)), eE = ldd(e + dindex(C, Ie, J));
   const df eS = ldd(e + dindex(C, I, Js)), eN = ldd(e + dindex(C, I, Jn));
-  const df c9 = add(scale2(e00, 0.5f), scale2(e00, 0.0625f));
+  const df c9 = df_nine(e00);
   const DBlk b = [&] {
     DBlk q;
     const int half = F.m >> 1;
@@ -343,9 +358,7 @@ __device__ __forceinline__ void df_prolong_plane(const DLev& C, const DLev& F, i
     return q;
   }();
   auto put = [&](int q, df x, df y, df xy) {
-    const df s = add(x, y);
-    const df v = sum4u(c9, scale2(s, 0.125f), scale2(s, 0.0625f), scale2(xy, 0.0625f));
-    F.d[c][b.in[q]] = f2(add(ldd(F.d[c] + b.in[q]), norm(v)));
+    F.d[c][b.in[q]] = f2(add(ldd(F.d[c] + b.in[q]), df_bilinear(c9, x, y, xy)));
   };
   put(0, eW, eS, ldd(e + dindex(C, Iw, Js)));
   put(1, eE, eS, ldd(e + dindex(C, Ie, Js)));

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "df_kernels.cuh"
+#include "df_leg.cuh"
 #include "mpfc_internal.h"
 
 using namespace mpfc;
@@ -200,6 +201,45 @@ int df_tail_first(const mpfc_s* H) {
   return lt;
 }
 
+// Levels that take one launch a way (df_leg.cuh): those of at most kLegCells cells above the
+// tail, with pre- and post-sweeps.  At 512^2 a launch's updates already take what the launch does and
+// the halo's only add to them: two steps at 1024^2 in 3.12 ms with that level too, 3.03 without; at
+// 512^2 3.04 and 2.84.
+constexpr long long kLegCells = 256 * 256;
+bool df_leg_level(const mpfc_s* H, int l) {
+  const int nu1 = H->p.nu1, nu2 = H->p.nu2, lt = df_tail_first(H);
+  return !df_unfused(H) && l < (lt < H->nlev ? lt : H->nlev - 1) && nu1 >= 1 && nu1 <= kLegMaxNu && nu2 >= 1 &&
+         nu2 <= kLegMaxNu && (long long)H->dlev[l].m * H->dlev[l].n <= kLegCells;
+}
+
+dim3 leg_grid(const DLev& L) { return dim3((L.m + kLegTile - 1) / kLegTile, (L.n + kLegTile - 1) / kLegTile); }
+
+template <int SCH>
+void launch_down(mpfc_s* H, const DPar& F, const DPar& C, bool first, cudaStream_t s) {
+  const size_t smem = leg_smem(H->p.nu1, SCH, F.L.W != nullptr, false);
+  auto go = [&](auto* k) { mpfc_launch(H->shape, k, leg_grid(F.L), dim3(kLegThreads), smem, s, F, C, H->p.nu1); };
+  if (F.L.nyn) go(first ? k_df_down<SCH, true, true> : k_df_down<SCH, true, false>);
+  else go(first ? k_df_down<SCH, false, true> : k_df_down<SCH, false, false>);
+}
+
+// The way up of level l; returns the level with its correction's planes.
+template <int SCH>
+DPar launch_up(mpfc_s* H, int l, const DPar& C, cudaStream_t s) {
+  DPar F = dpar(H, SCH, l);
+  LegOut O;
+  memset(&O, 0, sizeof(O));
+  for (int c = 0; c < 3; ++c) {
+    if (l == 0) O.u[c] = uplanes(H).u[c];
+    else O.e[c] = H->de[l][c];
+  }
+  const size_t smem = leg_smem(H->p.nu2, SCH, F.L.W != nullptr, true);
+  auto go = [&](auto* k) { mpfc_launch(H->shape, k, leg_grid(F.L), dim3(kLegThreads), smem, s, C, F, O, H->p.nu2); };
+  if (F.L.nyn) go(k_df_up<SCH, true>);
+  else go(k_df_up<SCH, false>);
+  for (int c = 0; c < 3; ++c) F.L.d[c] = O.e[c];
+  return F;
+}
+
 template <int SCH>
 void vcycle(mpfc_s* H, cudaStream_t s) {
   const mpfc_params& p = H->p;
@@ -209,6 +249,11 @@ void vcycle(mpfc_s* H, cudaStream_t s) {
   for (int l = 0; l < down; ++l) {
     MpfcRange range(mpfc_level_name(l));
     const DPar F = dpar(H, SCH, l), C = dpar(H, SCH, l + 1);
+    const bool first = (!unfused && !df_leg_level(H, l + 1)) || l + 1 == lt;   // the tail expects its first red sweep done
+    if (df_leg_level(H, l)) {
+      launch_down<SCH>(H, F, C, first, s);
+      continue;
+    }
     if (p.nu1 > 0) {
       if (unfused) launch_half<SCH, kAll, false>(H, F, 0, s);
       launch_half<SCH, kOwn, false>(H, F, 1, s);
@@ -218,14 +263,14 @@ void vcycle(mpfc_s* H, cudaStream_t s) {
     // the coarse level's correction starts at zero where no pre-smoothing forms it (the
     // coarsest solve writes all of it)
     const int zero = p.nu1 == 0 && l + 1 < L - 1;
-    const bool first = !unfused || l + 1 == lt;   // the tail expects its first red sweep done
     const dim3 g = mpfc_grid_of(sh, C.L.m, C.L.n), b = mpfc_blk_for(sh, C.L.m, C.L.n);
     if (unfused) {
       mpfc_launch(sh, k_df_base, g, b, 0, s, F, C);
       if (first) mpfc_launch(sh, k_df_restrict<SCH, true, false>, g, b, 0, s, F, C, zero);
       else mpfc_launch(sh, k_df_restrict<SCH, false, false>, g, b, 0, s, F, C, zero);
     } else {
-      mpfc_launch(sh, k_df_restrict<SCH, true, true>, g, b, 0, s, F, C, zero);
+      if (first) mpfc_launch(sh, k_df_restrict<SCH, true, true>, g, b, 0, s, F, C, zero);
+      else mpfc_launch(sh, k_df_restrict<SCH, false, true>, g, b, 0, s, F, C, zero);
     }
   }
   {
@@ -238,10 +283,16 @@ void vcycle(mpfc_s* H, cudaStream_t s) {
                   (const float*)H->K3[SCH - 1]);
     }
   }
+  DPar up = dpar(H, SCH, down);   // the level last finished, where its correction is
   for (int l = down - 1; l >= 0; --l) {
     MpfcRange range(mpfc_level_name(l));
-    const DPar F = dpar(H, SCH, l), C = dpar(H, SCH, l + 1);
+    if (df_leg_level(H, l)) {
+      up = launch_up<SCH>(H, l, up, s);
+      continue;
+    }
+    const DPar F = dpar(H, SCH, l), C = up;
     mpfc_launch(sh, k_df_prolong, mpfc_grid_of(sh, C.L.m, C.L.n), mpfc_blk_for(sh, C.L.m, C.L.n), 0, s, C, F);
+    up = F;
     for (int sw = 0; sw < p.nu2; ++sw)
       for (int color = 0; color < 2; ++color) {
         if (l == 0 && sw == p.nu2 - 1) launch_half<SCH, kGen, true>(H, F, color, s);
@@ -268,7 +319,7 @@ void defect(mpfc_s* H, int mode, cudaGraphConditionalHandle hnd, int set_cond, c
   A.zero = H->p.nu1 == 0;
   const dim3 g = pair_grid(H->p.m, H->p.n), b(32, 8);
   // the tail expects its first red sweep done, also where the finest level is in it
-  const bool first = !df_unfused(H) || df_tail_first(H) == 0;
+  const bool first = (!df_unfused(H) && !df_leg_level(H, 0)) || df_tail_first(H) == 0;
   if (mode == 0) {
     if (first) mpfc_launch(H->shape, k_df_defect<SCH, true, true>, g, b, 0, s, A);
     else mpfc_launch(H->shape, k_df_defect<SCH, true, false>, g, b, 0, s, A);
@@ -324,6 +375,11 @@ size_t mpfc_df_carve(mpfc_s* H, const mpfc_params* p, size_t* off, char* base, c
       }
       v.pb = reinterpret_cast<float2*>(lev[l].b1);
       v.pk = reinterpret_cast<float2*>(lev[l].b2);
+      if (H && base) {   // the way up's result (df_leg.cuh); the Poisson planes are mpfc_energy's
+        H->de[l][0] = reinterpret_cast<float2*>(lev[l].b3);
+        H->de[l][1] = reinterpret_cast<float2*>(px[l]);
+        H->de[l][2] = reinterpret_cast<float2*>(pf[l]);
+      }
     }
     if (H && base) H->dlev[l] = v;
   }
@@ -340,6 +396,22 @@ int mpfc_df_init(mpfc_s* H) {
   raise(k_df_tail<1, true>);
   raise(k_df_tail<2, false>);
   raise(k_df_tail<2, true>);
+  auto raise_leg = [&](auto* k, int scheme) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)leg_smem(kLegMaxNu, scheme, scheme == 2, true));
+  };
+  raise_leg(k_df_down<1, false, false>, 1);
+  raise_leg(k_df_down<1, false, true>, 1);
+  raise_leg(k_df_down<1, true, false>, 1);
+  raise_leg(k_df_down<1, true, true>, 1);
+  raise_leg(k_df_down<2, false, false>, 2);
+  raise_leg(k_df_down<2, false, true>, 2);
+  raise_leg(k_df_down<2, true, false>, 2);
+  raise_leg(k_df_down<2, true, true>, 2);
+  raise_leg(k_df_up<1, false>, 1);
+  raise_leg(k_df_up<1, true>, 1);
+  raise_leg(k_df_up<2, false>, 2);
+  raise_leg(k_df_up<2, true>, 2);
   if (e != cudaSuccess) {
     mpfc_set_cuda_error(e, "shared memory of the coarse tail", __FILE__, __LINE__);
     return MPFC_ERR_CUDA;
@@ -370,5 +442,7 @@ int mpfc_df_launches_per_cycle(const mpfc_s* H) {
   int per = 2 + 2 * nu2;                                           // restriction, prolongation, post-sweeps
   if (nu1 > 0) per += 2 * nu1 - 1 + (unfused ? 1 : 0);             // the first red half sweep is the producer's
   if (unfused) per += 1;                                           // p0 on its own
-  return down * per + 2 + ((down == 0 || nu2 == 0) ? 1 : 0);      // + tail or coarsest solve, + residual, (+ u += d)
+  int legs = 0;
+  for (int l = 0; l < down; ++l) legs += df_leg_level(H, l);
+  return (down - legs) * per + 2 * legs + 2 + ((down == 0 || nu2 == 0) ? 1 : 0);      // + tail or coarsest solve, + residual, (+ u += d)
 }

@@ -88,6 +88,7 @@ struct mpfc_s {
   cudaGraphConditionalHandle cur_handle = 0;   // handle of the graph being captured
   // correction form of the FP64 V-cycle (df_cycle.cu)
   mpfc::DLev dlev[mpfc::kMaxLevels];
+  float2* de[mpfc::kMaxLevels][3];   // coarse levels' corrections after a one-launch way up
   bool df = false;                               // the handle's V-cycles run in correction form
   cudaGraphConditionalHandle cur_handle64 = 0;   // loop of the FP64 V-cycle, for values outside the form's range
   int launch_mode = MPFC_LAUNCH_GRAPH;
