@@ -182,18 +182,18 @@ int mpfc_launch_counts(const mpfc_t* h, int scheme, int* per_step, int* per_cycl
  * The planes' contents change; call mpfc_set_state before stepping again. */
 int mpfc_fp32_time_smooth(mpfc_t* h, int level, int sweeps, float* ms);
 
-/* How the mixed-precision form's inner red-black sweeps run on levels launched per
- * level (a tuning choice: results do not depend on it, bit for bit).  tile_rows 0: each
- * sweep is two launches, one per colour, updating e in place.  tile_rows 4, 8, 16 or
- * 32: on levels of at least min_cells cells whose width is a multiple of 4, each sweep
- * is one launch over tiles of 64 x tile_rows cells staged in shared memory (e with a
- * two-cell halo), reading e from one copy in the workspace and writing the other, in
- * pairs so that e ends where it started.  Default: 16 rows on levels of at least
- * 2048 x 2048 cells, whose planes do not stay in L2 between sweeps (there the tiled
- * sweep reads each plane once instead of twice; smaller levels, served from L2, run
- * faster as two launches).  Drops
- * the handle's captured graphs.  MPFC_ERR_INVALID for other values or handles that are
- * not MPFC_FP32_INNER. */
+/* How the mixed-precision form's inner red-black sweeps run on levels of at least min_cells
+ * cells launched per level (a tuning choice: results do not depend on it, bit for bit).
+ * tile_rows 0: each sweep is two launches, one per colour, updating e in place.  tile_rows 4,
+ * 8, 16 or 32: where the width is a multiple of 4, each sweep is one launch over tiles of
+ * 64 x tile_rows cells staged in shared memory (e with a two-cell halo), reading e from
+ * one copy in the workspace and writing the other, in pairs so that e ends where it
+ * started.  Without this call, and on smaller levels, a level of a width that is a multiple
+ * of 4 takes one launch for its sweeps and the restriction and one for the prolongation and the
+ * sweeps (one or two sweeps of each kind), which is faster at every size; levels with other
+ * sweep counts run as with tile_rows 16 from 2048 x 2048 cells on and 0 below.  Drops the
+ * handle's captured graphs.  MPFC_ERR_INVALID for other values or handles that are not
+ * MPFC_FP32_INNER. */
 int mpfc_set_fp32_sweep(mpfc_t* h, int tile_rows, int min_cells);
 
 /* Test hook of the tiled FP32 sweep's failure handling (no counterpart in the paper; for

@@ -245,9 +245,11 @@ __device__ __forceinline__ void defect32(const Lev32& L, const Coef32& k, int i,
                 ld32<NC>(L.r3 + c), d1, d2, d3);
 }
 
-// coarse source = R(r - J e), coarse correction starts at zero
+// coarse source = R(r - J e), coarse correction starts at zero.  (cI, cJ): the coarse cell in C,
+// where F is a staged part of the fine level and (I, J) counts from its origin.
 template <bool NC>
-__device__ __forceinline__ void restrict_defect32_cell(const Lev32& F, const Lev32& C, const Coef32& kf, int I, int J) {
+__device__ __forceinline__ void restrict_defect32_cell(const Lev32& F, const Lev32& C, const Coef32& kf, int I, int J,
+                                                       int cI, int cJ) {
   float s1 = 0.f, s2 = 0.f, s3 = 0.f;
 #pragma unroll
   for (int dj = 0; dj < 2; ++dj)
@@ -259,7 +261,7 @@ __device__ __forceinline__ void restrict_defect32_cell(const Lev32& F, const Lev
       s2 += b;
       s3 += c;
     }
-  size_t cid = (size_t)J * C.m + I;
+  size_t cid = (size_t)cJ * C.m + cI;
   C.r1[cid] = 0.25f * s1;
   C.r2[cid] = 0.25f * s2;
   C.r3[cid] = 0.25f * s3;
@@ -273,12 +275,17 @@ __global__ void k_restrict_defect32(Lev32 F, Lev32 C, Coef32 kf) {
   int I = blockIdx.x * blockDim.x + threadIdx.x;
   int J = blockIdx.y * blockDim.y + threadIdx.y;
   if (I >= C.m || J >= C.n) return;
-  restrict_defect32_cell<true>(F, C, kf, I, J);
+  restrict_defect32_cell<true>(F, C, kf, I, J, I, J);
 }
 
 // e_f += P e_c (bilinear, shared-memory tiles of the three components of the coarse
 // correction, staged together)
 constexpr int kTX = 32, kTY = 8;
+// P e_c at a fine cell: its coarse cell, the neighbours on its side in x and y, the diagonal one
+__device__ __forceinline__ float prolonged32(float e00, float ex, float ey, float exy) {
+  const float w9 = 9.f / 16.f, w3 = 3.f / 16.f, w1 = 1.f / 16.f;
+  return fmaf(w3, ex + ey, fmaf(w1, exy, w9 * e00));
+}
 __device__ __forceinline__ void prolong32_apply(float (*E)[kTX + 2], float* __restrict__ ef, int mc, int I, int J) {
   int x = threadIdx.x + 1, y = threadIdx.y + 1;
   const float w9 = 9.f / 16.f, w3 = 3.f / 16.f, w1 = 1.f / 16.f;
@@ -878,6 +885,192 @@ void sweeps32(const mpfc_s* H, const Lev32& F, const Coef32& kf, const Coef32& k
   }
 }
 
+// ---------------------------------------------------------------------------
+// One level's way down or up of an inner V-cycle as one launch.  A CTA owns a tile of T x T
+// cells and sweeps it in shared memory with a halo: every half sweep needs the one before it on
+// one more ring of cells, which both tiles that hold it compute, from the same values with the
+// same cell functions (the bits are those of the per-level launches).  Every plane's lines
+// are read once a way instead of once a half sweep, and a level takes two launches instead of
+// ten.  Down: e (zero on coarse levels) from e's planes, the sweeps, the restriction, e to its
+// second copy; up: the prolongation onto that copy, the sweeps, e back to its own planes, so
+// no tile reads a halo that another one writes.  Bound by a tile's chain of phases (a way takes
+// 5.5 us from 64^2 to 256^2 and 11 at 512^2, against 11 to 25 for five launches) until the tiles fill
+// the chip, then by issue and shared memory: 30 us at 1024^2 (42), 95 to 110 at 2048^2 (97).
+// HX, HY: staged columns (whole 16-byte chunks: m is a multiple of 4) and rows around the tile.  The sweeps
+// and the restriction need 2 nu + 1 rings of e, but 2 nu where e is zero: the first half
+// sweep's neighbours are zeros wherever they are read (with Neumann rows two more, so that a
+// staged edge row that is swept is a boundary row).
+// ---------------------------------------------------------------------------
+constexpr int kLeg32MaxNu = 2;
+template <int T>
+constexpr int leg32_threads() { return T == 16 ? 288 : 512; }
+template <int T, int HX, int HY, bool UP>
+constexpr size_t leg32_smem() {
+  constexpr int cw = (T + 2 * HX) / 2 + 2, ch = (T + 2 * HY) / 2 + 2;
+  return sizeof(float) * (7 * (size_t)(T + 2 * HX) * (T + 2 * HY) + (UP ? 3 * cw * ch : 0));
+}
+
+template <int T, int HX, int HY>
+struct Leg32 {
+  static constexpr int W = T + 2 * HX, R = T + 2 * HY, P = W * R;
+  Lev32 S;              // the staged cells as a level of their own
+  int x0, y0, ylo;      // staged origin (x0 and ylo in the domain), the tile's first staged row
+  int bx, by;
+
+  __device__ __forceinline__ void init(const Lev32& F, float* sm) {
+    bx = blockIdx.x * T;
+    by = blockIdx.y * T;
+    ylo = by - HY;
+    int yhi = by + T + HY;
+    if (F.nyn) {   // no rows outside the domain: the staged edge row is the boundary row
+      ylo = max(ylo, 0);
+      yhi = min(yhi, F.n);
+    }
+    S = F;
+    S.m = W;
+    S.n = yhi - ylo;
+    S.ephi = sm;
+    S.emu = sm + P;
+    S.eka = sm + 2 * P;
+    S.r1 = sm + 3 * P;
+    S.r2 = sm + 4 * P;
+    S.r3 = sm + 5 * P;
+    S.q = sm + 6 * P;
+    y0 = by - ylo;
+    x0 = sw_col(bx - HX, F.m);
+    if (!F.nyn) ylo = sw_row(ylo, F.n, 0);
+  }
+  // Starts the copies of r and q, and of e from (e0, e1, e2) if OWN.
+  template <bool OWN>
+  __device__ __forceinline__ void load(const Lev32& F, const float* e0, const float* e1, const float* e2) const {
+    for (int t = threadIdx.x; t < S.n * (W / 4); t += blockDim.x) {
+      const int r = t / (W / 4), c = 4 * (t - r * (W / 4));
+      int x = x0 + c, y = ylo + r;
+      x = x < F.m ? x : x % F.m;
+      if (y >= F.n) y %= F.n;
+      const size_t g = (size_t)y * F.m + x;
+      const int d = r * W + c;
+      cp_async16(S.r1 + d, F.r1 + g);
+      cp_async16(S.r2 + d, F.r2 + g);
+      cp_async16(S.r3 + d, F.r3 + g);
+      cp_async16(S.q + d, F.q + g);
+      if (OWN) {
+        cp_async16(S.ephi + d, e0 + g);
+        cp_async16(S.emu + d, e1 + g);
+        cp_async16(S.eka + d, e2 + g);
+      }
+    }
+    cp_async_commit();
+  }
+  // Half sweep of colour `color` on the tile and `ring` rings around it.
+  __device__ __forceinline__ void half_sweep(const Coef32& k, const Coef32& kb, int color, int ring) const {
+    int lo = y0 - ring, hi = y0 + T + ring;
+    if (S.nyn) {
+      lo = max(lo, 0);
+      hi = min(hi, S.n);
+    }
+    const int per = T / 2 + ring, inv = 65536 / per + 1;   // t / per = t inv >> 16 for t < 65536 / per
+    for (int t = threadIdx.x; t < (hi - lo) * per; t += blockDim.x) {
+      const int r = (t * inv) >> 16, j = lo + r, par = (j + color) & 1;
+      smooth32_cell<false>(S, k, kb, 2 * (((HX - ring + 1 - par) >> 1) + t - r * per) + par, j);
+    }
+    __syncthreads();
+  }
+  // The tile's e to planes of the level, by the threads from `first` on.
+  __device__ __forceinline__ void store(const Lev32& F, float* e0, float* e1, float* e2, int first) const {
+    for (int t = threadIdx.x - first; t < T * T / 4; t += blockDim.x - first) {
+      const int r = t / (T / 4), c = 4 * (t - r * (T / 4));
+      if (bx + c >= F.m || by + r >= F.n) continue;
+      const size_t g = (size_t)(by + r) * F.m + bx + c;
+      const int q = (y0 + r) * W + HX + c;
+      *reinterpret_cast<float4*>(e0 + g) = *reinterpret_cast<const float4*>(S.ephi + q);
+      *reinterpret_cast<float4*>(e1 + g) = *reinterpret_cast<const float4*>(S.emu + q);
+      *reinterpret_cast<float4*>(e2 + g) = *reinterpret_cast<const float4*>(S.eka + q);
+    }
+  }
+};
+
+template <int T, int HX, int HY, bool ZERO>
+__global__ void __launch_bounds__(leg32_threads<T>()) k_leg32_down(Lev32 F, Lev32 C, Coef32 kf, Coef32 kb, int nu) {
+  extern __shared__ __align__(16) float l32[];
+  Leg32<T, HX, HY> G;
+  G.init(F, l32);
+  pdl_enter();
+  G.template load<!ZERO>(F, F.ephi, F.emu, F.eka);
+  if (ZERO)
+    for (int t = threadIdx.x; t < 3 * G.P; t += blockDim.x) l32[t] = 0.f;
+  cp_async_wait_all();
+  __syncthreads();
+  for (int hs = 0; hs < 2 * nu; ++hs) G.half_sweep(kf, kb, hs & 1, 2 * nu - hs);
+  constexpr int kRw = T * T / 4;   // the first warps restrict while the others store e
+  if (threadIdx.x < kRw) {
+    const int I = threadIdx.x % (T / 2), J = threadIdx.x / (T / 2), cI = G.bx / 2 + I, cJ = G.by / 2 + J;
+    if (cI < C.m && cJ < C.n) restrict_defect32_cell<false>(G.S, C, kf, HX / 2 + I, G.y0 / 2 + J, cI, cJ);
+  } else {
+    G.store(F, F.xphi, F.xmu, F.xka, kRw);
+  }
+}
+
+// r, q and the second copy of e were written before the previous launch, whose start waited for
+// them: they are read before the wait for the coarse level's correction.
+template <int T>
+__global__ void __launch_bounds__(leg32_threads<T>()) k_leg32_up(Lev32 C, Lev32 F, Coef32 kf, Coef32 kb, int nu) {
+  constexpr int H = 4;
+  extern __shared__ __align__(16) float l32[];
+  Leg32<T, H, H> G;
+  G.init(F, l32);
+  G.template load<true>(F, F.xphi, F.xmu, F.xka);
+  pdl_enter();
+  constexpr int cw = G.W / 2 + 2, CP = cw * (G.R / 2 + 2);
+  float* const e = l32 + 7 * G.P;   // the coarse correction under the staged cells with one ring
+  for (int t = threadIdx.x; t < cw * (G.S.n / 2 + 2); t += blockDim.x) {
+    const int r = t / cw, I = sw_col(G.x0 / 2 - 1 + t - r * cw, C.m), J = sw_row(G.ylo / 2 - 1 + r, C.n, C.nyn);
+    const size_t g = (size_t)J * C.m + I;
+    e[t] = C.ephi[g];
+    e[CP + t] = C.emu[g];
+    e[2 * CP + t] = C.eka[g];
+  }
+  cp_async_wait_all();
+  __syncthreads();
+  for (int t = threadIdx.x; t < G.W * G.S.n; t += blockDim.x) {
+    const int j = t / G.W, i = t - j * G.W;
+    const float* f = e + ((j >> 1) + 1) * cw + (i >> 1) + 1;
+    const int dx = (i & 1) ? 1 : -1, dy = (j & 1) ? cw : -cw;
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      l32[c * G.P + t] += prolonged32(f[c * CP], f[c * CP + dx], f[c * CP + dy], f[c * CP + dx + dy]);
+  }
+  __syncthreads();
+  for (int hs = 0; hs < 2 * nu; ++hs) G.half_sweep(kf, kb, hs & 1, 2 * nu - 1 - hs);
+  G.store(F, F.ephi, F.emu, F.eka, 0);
+}
+
+// Levels that take one launch a way: those with a second copy of e and one or two sweeps of
+// each kind, unless mpfc_set_fp32_sweep was called for levels of their size.
+// Four mixed steps at 1024^2 in 4.22 ms against 4.77 with the per-level launches, at 512 x 384 in
+// 2.16 against 2.90, at 2048^2 in 11.6 against 11.85 (there with the one-launch sweeps).  Tiles of
+// 32 x 32 cells have less halo (1.2 times the updates, 1.43 with 16 x 16) but are too few for the
+// chip on a small level: 16 x 16 on every level makes 1024^2 4.60 ms and 2048^2 13.7.
+constexpr long long kLeg32Small = 256 * 256;   // levels of at most this many cells: 16 x 16 tiles
+bool leg32_level(const mpfc_s* H, const Lev32& F) {
+  const int nu1 = H->p.nu1, nu2 = H->p.nu2;
+  return F.xphi && nu1 >= 1 && nu1 <= kLeg32MaxNu && nu2 >= 1 && nu2 <= kLeg32MaxNu && !(H->sweep_set && (long long)F.m * F.n >= H->sweep_tile_cells);
+}
+
+template <int T>
+void leg32_down(mpfc_s* H, const Lev32& F, const Lev32& C, const Coef32& kf, const Coef32& kb, bool zero, cudaStream_t s) {
+  const dim3 g((F.m + T - 1) / T, (F.n + T - 1) / T), b(leg32_threads<T>());
+  if (zero && F.nyn)
+    mpfc_launch(H->shape, k_leg32_down<T, 4, 6, true>, g, b, leg32_smem<T, 4, 6, false>(), s, F, C, kf, kb, H->p.nu1);
+  else if (zero) mpfc_launch(H->shape, k_leg32_down<T, 4, 4, true>, g, b, leg32_smem<T, 4, 4, false>(), s, F, C, kf, kb, H->p.nu1);
+  else mpfc_launch(H->shape, k_leg32_down<T, 8, 6, false>, g, b, leg32_smem<T, 8, 6, false>(), s, F, C, kf, kb, H->p.nu1);
+}
+template <int T>
+void leg32_up(mpfc_s* H, const Lev32& C, const Lev32& F, const Coef32& kf, const Coef32& kb, cudaStream_t s) {
+  mpfc_launch(H->shape, k_leg32_up<T>, dim3((F.m + T - 1) / T, (F.n + T - 1) / T), dim3(leg32_threads<T>()),
+              leg32_smem<T, 4, 4, true>(), s, C, F, kf, kb, H->p.nu2);
+}
+
 int inner_cycles_of(const mpfc_s* H) { return H->p.inner_cycles > 0 ? H->p.inner_cycles : 2; }
 
 // ---------------------------------------------------------------------------
@@ -905,9 +1098,7 @@ __device__ __forceinline__ void prolong32_fine(const float* ec, float* ef, int m
   const int I = fi >> 1, J = fj >> 1;
   const int Ix = wrapm(I + ((fi & 1) ? 1 : -1), mc), Jy = ywrap(J + ((fj & 1) ? 1 : -1), nc, nyn);
   const float e00 = ec[J * mc + I], ex = ec[J * mc + Ix], ey = ec[Jy * mc + I], exy = ec[Jy * mc + Ix];
-  const float w9 = 9.f / 16.f, w3 = 3.f / 16.f, w1 = 1.f / 16.f;
-  const int id = fj * (2 * mc) + fi;
-  ef[id] += fmaf(w3, ex + ey, fmaf(w1, exy, w9 * e00));
+  ef[fj * (2 * mc) + fi] += prolonged32(e00, ex, ey, exy);
 }
 
 size_t tail32_smem(const Lev32* levs, int nlev) {
@@ -992,7 +1183,10 @@ __global__ void __launch_bounds__(kTail32Threads) k_tail32(const __grid_constant
       __syncthreads();
     }
     if (!up) {
-      for (int t = tid; t < cc; t += nt) restrict_defect32_cell<false>(F, C, A.k[l], t % C.m, t / C.m);
+      for (int t = tid; t < cc; t += nt) {
+        const int I = t % C.m, J = t / C.m;
+        restrict_defect32_cell<false>(F, C, A.k[l], I, J, I, J);
+      }
       __syncthreads();
       if (l + 1 == down) {
         coarse32_block(sl[down], A.k[down], k3s, scratch);
@@ -1050,6 +1244,11 @@ void enqueue_inner_vcycle(mpfc_s* H, int scheme, cudaStream_t s) {
     const Lev32& F = H->lev32[l];
     const Lev32& C = H->lev32[l + 1];
     Coef32 kf = coef32_of(H->coef[scheme - 1][l]), kb = coef32_of(H->coefb[scheme - 1][l]);
+    if (leg32_level(H, F)) {
+      if ((long long)F.m * F.n <= kLeg32Small) leg32_down<16>(H, F, C, kf, kb, l > 0, s);
+      else leg32_down<32>(H, F, C, kf, kb, l > 0, s);
+      continue;
+    }
     sweeps32(H, F, kf, kb, p.nu1, s);
     mpfc_launch(sh, k_restrict_defect32, mpfc_grid_of(sh, C.m, C.n), mpfc_blk_for(sh, C.m, C.n), 0, s, F, C, kf);
   }
@@ -1064,6 +1263,11 @@ void enqueue_inner_vcycle(mpfc_s* H, int scheme, cudaStream_t s) {
     const Lev32& F = H->lev32[l];
     const Lev32& C = H->lev32[l + 1];
     Coef32 kf = coef32_of(H->coef[scheme - 1][l]), kb = coef32_of(H->coefb[scheme - 1][l]);
+    if (leg32_level(H, F)) {
+      if ((long long)F.m * F.n <= kLeg32Small) leg32_up<16>(H, C, F, kf, kb, s);
+      else leg32_up<32>(H, C, F, kf, kb, s);
+      continue;
+    }
     mpfc_launch(sh, k_prolong32, grid_of(C.m, C.n), kBlk, 0, s, F, C);
     sweeps32(H, F, kf, kb, p.nu2, s);
   }
@@ -1156,6 +1360,7 @@ extern "C" int mpfc_set_fp32_sweep(mpfc_t* H, int tile_rows, int min_cells) {
     return MPFC_ERR_INVALID;
   H->sweep_tile_rows = tile_rows;
   H->sweep_tile_cells = min_cells;
+  H->sweep_set = true;
   mpfc_drop_graphs(H);
   return MPFC_OK;
 }
@@ -1190,6 +1395,15 @@ int mpfc_fp32_init(mpfc_s* H) {
   H->K3f[0] = H->K3[0];
   H->K3f[1] = H->K3[1];
   cudaError_t e = cudaFuncSetAttribute(k_tail32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTail32MaxSmem);
+  auto raise = [&](auto* k, size_t smem) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  };
+  raise(k_leg32_down<16, 8, 6, false>, leg32_smem<16, 8, 6, false>());
+  raise(k_leg32_down<32, 4, 6, true>, leg32_smem<32, 4, 6, false>());
+  raise(k_leg32_down<32, 4, 4, true>, leg32_smem<32, 4, 4, false>());
+  raise(k_leg32_down<32, 8, 6, false>, leg32_smem<32, 8, 6, false>());
+  raise(k_leg32_up<16>, leg32_smem<16, 4, 4, true>());
+  raise(k_leg32_up<32>, leg32_smem<32, 4, 4, true>());
   if (e != cudaSuccess) {
     mpfc_set_cuda_error(e, "shared memory of the FP32 tail kernel", __FILE__, __LINE__);
     return MPFC_ERR_CUDA;

@@ -103,6 +103,7 @@ struct mpfc_s {
   float* K3f[2] = {nullptr, nullptr};
   int sweep_tile_rows = 16;                     // FP32 one-launch sweeps: tile height (0: two launches per sweep)
   long long sweep_tile_cells = 2048LL * 2048;   // ... on levels of at least this many cells
+  bool sweep_set = false;                       // mpfc_set_fp32_sweep was called: levels of that size take those sweeps
   int outer_max = 0;
   // learned initial guess
   MpfcGuess guess;
