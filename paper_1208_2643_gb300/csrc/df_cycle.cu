@@ -342,11 +342,11 @@ bool mpfc_df_usable(const mpfc_s* H) {
   return true;
 }
 
-// Planes of the correction form.  Level 0: corrections and rho in memory of their own, p0
-// and phi^k in the Poisson planes (used only by mpfc_energy); coarser levels in the FP64
-// V-cycle's planes, which it writes before it reads them.
-size_t mpfc_df_carve(mpfc_s* H, const mpfc_params* p, size_t* off, char* base, const Lev* lev, double* const* px,
-                     double* const* pf, int nlev) {
+// Planes of the correction form.  Level 0: corrections and rho in dr0, p0 and phi^k in the
+// Poisson planes (used only by mpfc_energy); coarser levels in the FP64 V-cycle's planes, which
+// it writes before it reads them, and a one-launch way up's result in planes of its own.
+size_t mpfc_df_carve(mpfc_s* H, const mpfc_params* p, size_t* off, char* base, const Lev* lev, double* const* dr0,
+                     double* px0, double* pf0, int nlev) {
   if (p->precision != MPFC_FP64 || nlev < 2) return 0;
   const size_t start = *off;
   auto take = [&](size_t cells) -> float2* {
@@ -362,10 +362,12 @@ size_t mpfc_df_carve(mpfc_s* H, const mpfc_params* p, size_t* off, char* base, c
     v.W = nullptr;
     const size_t G = (size_t)v.m * v.n;
     if (l == 0) {
-      for (int c = 0; c < 3; ++c) v.d[c] = take(G);
-      for (int c = 0; c < 3; ++c) v.r[c] = take(G);
-      v.pb = reinterpret_cast<float2*>(px[0]);
-      v.pk = reinterpret_cast<float2*>(pf[0]);
+      for (int c = 0; c < 3; ++c) {
+        v.d[c] = reinterpret_cast<float2*>(dr0[c]);
+        v.r[c] = reinterpret_cast<float2*>(dr0[3 + c]);
+      }
+      v.pb = reinterpret_cast<float2*>(px0);
+      v.pk = reinterpret_cast<float2*>(pf0);
     } else {
       double* const d[3] = {lev[l].phi, lev[l].mu, lev[l].ka};
       double* const r[3] = {lev[l].S1, lev[l].S2, lev[l].S3};
@@ -375,10 +377,9 @@ size_t mpfc_df_carve(mpfc_s* H, const mpfc_params* p, size_t* off, char* base, c
       }
       v.pb = reinterpret_cast<float2*>(lev[l].b1);
       v.pk = reinterpret_cast<float2*>(lev[l].b2);
-      if (H && base) {   // the way up's result (df_leg.cuh); the Poisson planes are mpfc_energy's
-        H->de[l][0] = reinterpret_cast<float2*>(lev[l].b3);
-        H->de[l][1] = reinterpret_cast<float2*>(px[l]);
-        H->de[l][2] = reinterpret_cast<float2*>(pf[l]);
+      for (int c = 0; c < 3; ++c) {
+        float2* e = (long long)G <= kLegCells ? take(G) : nullptr;
+        if (H && base) H->de[l][c] = e;
       }
     }
     if (H && base) H->dlev[l] = v;

@@ -209,6 +209,20 @@ static size_t carve(mpfc_s* H, const mpfc_params* p, char* base) {
   double h = p->h;
   Lev lev[kMaxLevels];
   double *px[kMaxLevels], *pf[kMaxLevels], *pw[kMaxLevels];
+  // The finest level's d and rho of the correction form; the coarse levels' planes that are dead
+  // while it runs (kept R kappa_f and phi^k of the FP64 V-cycle, the energies' Poisson planes)
+  // share their memory.
+  const bool dfp = p->precision == MPFC_FP64 && L >= 2;
+  double* dr0[6] = {};
+  const size_t dr_off = c.off;
+  if (dfp)
+    for (int k = 0; k < 6; ++k) dr0[k] = c.take<double>(G0);
+  const size_t dr_end = c.off;
+  Carver shared{base, dr_off};
+  auto dead = [&](size_t G) {
+    if (dfp && align256(shared.off + G * sizeof(double)) <= dr_end) return shared.take<double>(G);
+    return c.take<double>(G);
+  };
   for (int l = 0; l < L; ++l) {
     size_t G = (size_t)m * n;
     Lev& v = lev[l];
@@ -226,14 +240,14 @@ static size_t carve(mpfc_s* H, const mpfc_params* p, char* base) {
     if (l > 0) {
       v.b1 = c.take<double>(G);
       v.b2 = c.take<double>(G);
-      v.b3 = c.take<double>(G);
-      v.pk = c.take<double>(G);
+      v.b3 = dead(G);
+      v.pk = dead(G);
     } else {
       v.b1 = v.b2 = v.b3 = nullptr;
       v.pk = phik;
     }
-    px[l] = c.take<double>(G);
-    pf[l] = c.take<double>(G);
+    px[l] = l > 0 ? dead(G) : c.take<double>(G);
+    pf[l] = l > 0 ? dead(G) : c.take<double>(G);
     pw[l] = p->pinning ? c.take<double>(G) : nullptr;
     m /= 2;
     n /= 2;
@@ -245,7 +259,7 @@ static size_t carve(mpfc_s* H, const mpfc_params* p, char* base) {
   float* K3b = c.take<float>(2 * (size_t)Gc * Gc);
   float* poisP = c.take<float>((size_t)Gc * Gc);
   mpfc_fp32_carve(H, p, &c.off, base, L);
-  mpfc_df_carve(H, p, &c.off, base, lev, px, pf, L);
+  mpfc_df_carve(H, p, &c.off, base, lev, dr0, px[0], pf[0], L);
   mpfc_guess_carve(H, p, &c.off, base);
   if (H && base) {
     H->nlev = L;
@@ -706,8 +720,19 @@ static void learned_body(mpfc_s* H, int scheme, cudaStream_t s) {
   else enqueue_learned_correction<2>(H, H->cur_handle, 1, s);
 }
 
+// phi^k on the coarse levels in FP64, for a V-cycle after the correction form's: it shares memory
+// with that form's planes (carve).
+static void enqueue_coarse_phik(mpfc_s* H, cudaStream_t s) {
+  for (int l = 1; l < H->nlev; ++l) {
+    const Lev& C = H->lev[l];
+    mpfc_launch(H->shape, k_restrict_plane, grid_for(C.m, C.n, kBlk2d), kBlk2d, 0, s, (const double*)H->lev[l - 1].pk, C.pk,
+                C.m, C.n);
+  }
+}
+
 static void fp64_body(mpfc_s* H, int scheme, cudaStream_t s) {
   cudaGraphConditionalHandle hnd = H->cur_handle;
+  if (scheme == 2 && H->df) enqueue_coarse_phik(H, s);
   if (scheme == 1) {
     enqueue_vcycle<1>(H, s);
     enqueue_resnorm<1>(H, 1, hnd, 1, s);
@@ -871,6 +896,7 @@ static int step_stream_mode(mpfc_s* H, int scheme) {
       mpfc_df_defect(H, scheme, 1, 0, 0, s);
       continue;
     }
+    if (scheme == 2 && H->df) enqueue_coarse_phik(H, s);
     if (scheme == 1) {
       enqueue_vcycle<1>(H, s);
       enqueue_resnorm<1>(H, 1, 0, 0, s);

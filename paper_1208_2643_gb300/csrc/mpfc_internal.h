@@ -184,8 +184,8 @@ void mpfc_enqueue_commit(mpfc_s* H, int scheme, cudaStream_t s);
 int mpfc_tail_first_level(const mpfc_s* H);
 
 // correction form of the FP64 V-cycle (df_cycle.cu)
-size_t mpfc_df_carve(mpfc_s* H, const mpfc_params* p, size_t* off, char* base, const mpfc::Lev* lev, double* const* px,
-                     double* const* pf, int nlev);
+size_t mpfc_df_carve(mpfc_s* H, const mpfc_params* p, size_t* off, char* base, const mpfc::Lev* lev,
+                     double* const* dr0, double* px0, double* pf0, int nlev);
 bool mpfc_df_usable(const mpfc_s* H);
 int mpfc_df_init(mpfc_s* H);
 void mpfc_df_restrict_pk(mpfc_s* H, int l, cudaStream_t s);
