@@ -334,7 +334,8 @@ void mpfc_build_K3(const Lev& C, const Coef& k, std::vector<double>& K3) {
 //     1024^2 in 3.62 ms against 4.24 (one-warp blocks), 3.67 (32 x 2) and 3.75 (32 x 8),
 //     one step at 4096^2 in 16.9 ms against 22.4, 17.1 and 17.3; programmatic launch for
 //     every grid costs 3 % at 4096^2.  The levels of at most 16 x 16 cells as one
-//     single-CTA launch (32 x 32: 3.60 ms at 1024^2; 64 x 64: 3.96).
+//     single-CTA launch: with the levels above it in one launch a way, two steps at 1024^2 in
+//     3.03 ms against 3.06 (8 x 8) and 3.10 (32 x 32), four at 512^2 in 2.84, 2.87 and 2.94.
 //   The FP64 V-cycle (outside the correction form's range only) prefers one-warp blocks and
 //     programmatic launch up to 128 blocks: 2.92 against 3.7 ms per step at 1024^2.
 mpfc_launch_shape mpfc_default_launch_shape(int precision) {
