@@ -23,6 +23,12 @@ struct DSum {
   double d;
   df f;
 };
+// Norms for which the scaled squares of the next residual keep their low parts in binary32: from
+// kDfMinResidual up to far below what a residual value may be (df_of keeps 48 bits to 2^99).
+// Zero, infinities and NaN are not among them.
+__device__ __forceinline__ bool df_norm_in_range(double res) {
+  return f64_exp(res) - (1023u - 56u) <= 56u + 60u;
+}
 __device__ __forceinline__ float df_norm_scale(double res) {
   const unsigned e = f64_exp(res);
   return (e < 1023u - 100u || e > 1023u + 100u) ? 1.0f : __uint_as_float((127u + 1023u - e) << 23);

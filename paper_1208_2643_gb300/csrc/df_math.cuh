@@ -95,14 +95,14 @@ __device__ __forceinline__ df lap5(df w, df e, df s, df n, df c) {
 
 // binary64 -> float-float: the high part truncated (integer pipes), the 29 significand
 // bits below it as the low part (converted to binary32: 24 of them, so 48 bits in all).
-// Zero and magnitudes below 2^-74 (whose low part's scale leaves the normal binary32 range)
-// keep the high part only; callers keep magnitudes far below 2^100.
+// Zero, magnitudes below 2^-74 (whose low part's scale leaves the normal binary32 range) and
+// from 2^100 on keep one part only, the value rounded to nearest.
 __device__ __forceinline__ df df_of(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const unsigned int hi = (unsigned int)(b >> 32), eb = (hi >> 20) & 0x7FFu;
   if (eb - (1023u - 74u) >= 174u) {
     if ((b << 1) == 0ull) return df{0.0f, 0.0f};
-    return df{f64_to_f32_trunc(x), 0.0f};
+    return df{f64_to_f32_rn(x), 0.0f};
   }
   const unsigned int sg = hi & 0x80000000u, ef = (eb - 1023u + 127u) << 23;
   // low 29 bits times 2^(e - 52), with the sign of x

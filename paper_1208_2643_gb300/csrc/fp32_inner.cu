@@ -59,14 +59,16 @@ dim3 grid_of(int X, int Y) { return dim3((X + kBlk.x - 1) / kBlk.x, (Y + kBlk.y 
 // e = 0, and the scaled residual norm with the outer loop decision.  Bound by the FP64 pipe
 // (8 instructions a cell in scheme 1, the Laplacians being integer sums, lap5_f64); the
 // linearisation and, after the first cycle, the squares are float-float (as in
-// df_defect_pair): 40 us at 1024^2, 75 with all of it in FP64.
+// df_defect_pair): 40 us at 1024^2, 75 with all of it in FP64.  The squares are FP64 too where
+// the last norm says that binary32 could lose them (df_norm_in_range).
 // ---------------------------------------------------------------------------
 template <int SCH>
 __global__ void __launch_bounds__(256, 5) k_defect(Lev L, Coef k, Lev32 E, Ctl* ctl, double* partials, int mode,
                                                 cudaGraphConditionalHandle hnd, int set_cond) {
   pdl_enter();
   DSum sum{0.0, df{0.f, 0.f}};
-  const float scale = mode == 0 ? 1.0f : df_norm_scale(ctl->res);
+  const bool wide = mode == 0 || !df_norm_in_range(ctl->res);
+  const float scale = wide ? 1.0f : df_norm_scale(ctl->res);
   const df gam = df_of(k.gam);
   const int half = L.m >> 1;
   for (int j = blockIdx.y * blockDim.y + threadIdx.y; j < L.n; j += gridDim.y * blockDim.y)
@@ -79,7 +81,7 @@ __global__ void __launch_bounds__(256, 5) k_defect(Lev L, Coef k, Lev32 E, Ctl* 
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const df r1 = df_of(R.a[c]), r2 = df_of(R.b[c]), r3 = df_of(R.c[c]);
-        if (mode == 0) sum.d = fma(R.a[c], R.a[c], fma(R.b[c], R.b[c], fma(R.c[c], R.c[c], sum.d)));
+        if (wide) sum.d = fma(R.a[c], R.a[c], fma(R.b[c], R.b[c], fma(R.c[c], R.c[c], sum.d)));
         else sum.f = add(sum.f, df_squares(r1, r2, r3, scale));
         o1[c] = fadd(r1.h, r1.l);
         o2[c] = fadd(r2.h, r2.l);
@@ -100,7 +102,7 @@ __global__ void __launch_bounds__(256, 5) k_defect(Lev L, Coef k, Lev32 E, Ctl* 
       put(E.emu, 0.f, 0.f);
       put(E.eka, 0.f, 0.f);
     }
-  double v[1] = {mode == 0 ? df_warp_sum<true>(sum, scale) : df_warp_sum<false>(sum, scale)};
+  double v[1] = {wide ? df_warp_sum<true>(sum, scale) : df_warp_sum<false>(sum, scale)};
   if (!grid_sum<1, true>(v, partials, &ctl->counter)) return;
   double res = sqrt(v[0] / (3.0 * (double)(L.m * L.n)));
   int cond;
