@@ -186,9 +186,10 @@ __global__ void __launch_bounds__(256) k_pois_apply(const __grid_constant__ DLev
 }
 
 // x = 0, f = rhs - mean; sums: 1 sum f^2, 2 cycles (0), 3 the power of two nearest below
-// 1 / rms(f), by which F is scaled into the middle of the binary32 range, and 4 its inverse.
+// 1 / rms(h^2 f), by which F is scaled into the middle of the binary32 range, and 4 its inverse.
 __global__ void __launch_bounds__(256) k_pois_start(const double* __restrict__ rhs, double* __restrict__ f,
-                                                    double* __restrict__ x, int G, Ctl* ctl, double* partials) {
+                                                    double* __restrict__ x, int G, double h2, Ctl* ctl,
+                                                    double* partials) {
   pdl_enter();
   const double mean = ctl->sums[0] / (double)G;
   double v[1] = {0.0};
@@ -199,7 +200,8 @@ __global__ void __launch_bounds__(256) k_pois_start(const double* __restrict__ r
     v[0] = fma(r, r, v[0]);
   }
   if (!grid_sum<1>(v, partials, &ctl->counter)) return;
-  const int e = (v[0] > 0.0 && !isinf(v[0])) ? ilogb(sqrt(v[0] / (double)G)) : 0;
+  const double rms = h2 * sqrt(v[0] / (double)G);
+  const int e = rms > 0.0 && !isinf(rms) ? min(max(ilogb(rms), -1000), 1000) : 0;
   ctl->sums[0] = v[0];
   ctl->sums[1] = v[0];
   ctl->sums[2] = 0.0;
@@ -380,7 +382,8 @@ int mpfc_pois_solve(mpfc_s* H) {
     const dim3 g(mpfc_reduce_blocks((size_t)G)), b(256);
     const double h = H->lev[0].h;
     mpfc_launch(sh, k_sum1, g, b, 0, cs, (const double*)H->psik, G, H->ctl, H->partials);
-    mpfc_launch(sh, k_pois_start, g, b, 0, cs, (const double*)H->psik, H->pf[0], H->px[0], G, H->ctl, H->partials);
+    mpfc_launch(sh, k_pois_start, g, b, 0, cs, (const double*)H->psik, H->pf[0], H->px[0], G, h * h, H->ctl,
+                H->partials);
     mpfc_launch(sh, k_pois_resid<true>, g, b, 0, cs, (const double*)H->px[0], (const double*)H->pf[0], plev(H, 0), h * h,
                 1.0 / (h * h), H->ctl, H->partials, hnd);
     H->cur_handle = hnd;
