@@ -196,7 +196,7 @@ void launch_df_tail(mpfc_s* H, int lt, cudaStream_t s) {
 }
 
 int df_tail_first(const mpfc_s* H) {
-  int lt = mpfc_tail_first_level(H);
+  int lt = mpfc_tail_first_level(H, H->shape);
   if (lt < H->nlev && H->nlev - lt > kDfTailMax) lt = H->nlev - kDfTailMax;
   return lt;
 }

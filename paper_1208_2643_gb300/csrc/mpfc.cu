@@ -336,13 +336,15 @@ void mpfc_build_K3(const Lev& C, const Coef& k, std::vector<double>& K3) {
 //     every grid costs 3 % at 4096^2.  The levels of at most 16 x 16 cells as one
 //     single-CTA launch: with the levels above it in one launch a way, two steps at 1024^2 in
 //     3.03 ms against 3.06 (8 x 8) and 3.10 (32 x 32), four at 512^2 in 2.84, 2.87 and 2.94.
-//   The FP64 V-cycle (outside the correction form's range only) prefers one-warp blocks and
-//     programmatic launch up to 128 blocks: 2.92 against 3.7 ms per step at 1024^2.
-mpfc_launch_shape mpfc_default_launch_shape(int precision) {
-  if (precision == MPFC_FP32_INNER) return mpfc_launch_shape{4, 0, 4 * mpfc::sm_count(), 32 * 32, 1, 0};
-  // split transfers of the FP64 V-cycle up to 256^2 fine cells: 2.917 against 2.975 ms per
-  // step at 1024^2 without, with one-warp blocks
-  return mpfc_launch_shape{4, 0, 4 * mpfc::sm_count(), 256, 1, 256 * 256};
+//   The FP64 V-cycle (outside the correction form's range), bound by the FP64 pipe: one-warp
+//     blocks and programmatic launch up to 128 blocks.  A step of six V-cycles at 512^2 in
+//     1.98 ms against 2.15 with the shape above, at 1024^2 in 4.35 against 4.50, at 2048^2 in 13.2
+//     against 13.4 (at 128^2 in 1.11 against 1.08); the block's rows alone are worth 0.5 %.
+// df: for kernels around the correction form; false: for FP64 V-cycles.
+mpfc_launch_shape mpfc_default_launch_shape(int precision, bool df) {
+  const int four = 4 * mpfc::sm_count();
+  if (precision == MPFC_FP32_INNER) return mpfc_launch_shape{4, 0, four, 32 * 32, 1, 0};
+  return mpfc_launch_shape{df ? 4 : 1, 0, df ? four : 128, 256, 1, 256 * 256};
 }
 
 // The coarsest grid's matrices for one scheme as the FP32 block the coarse solves read:
@@ -374,7 +376,6 @@ extern "C" int mpfc_create(const mpfc_params* p, void* d_workspace, size_t bytes
   if (!d_workspace || bytes < need || ((uintptr_t)d_workspace & 255)) return MPFC_ERR_WORKSPACE;
   mpfc_s* H = new mpfc_s();
   H->p = *p;
-  H->shape = mpfc_default_launch_shape(p->precision);
   H->guess_gate = kGuessGateTolMultiple * p->tol;
   H->stream = (cudaStream_t)cuda_stream;
   H->ws = (char*)d_workspace;
@@ -386,6 +387,8 @@ extern "C" int mpfc_create(const mpfc_params* p, void* d_workspace, size_t bytes
       H->coefb[s][l] = mpfc_coef(p, s + 1, H->lev[l].h, 3);
     }
   H->df = mpfc_df_usable(H);
+  H->shape = mpfc_default_launch_shape(p->precision, H->df);
+  H->shape64 = mpfc_default_launch_shape(p->precision, false);
   int rc = MPFC_OK;
   do {
     cudaError_t e;
@@ -522,17 +525,17 @@ int mpfc_tail_max_ctas() {
 
 template <int SCH>
 static void launch_coarse(mpfc_s* H, const Lev& C, const Coef& k, cudaStream_t s) {
-  mpfc_launch(H->shape, k_coarse_solve<SCH>, dim3(1), dim3(32), coarse_smem(C), s, C, k, (const float*)H->K3[SCH - 1]);
+  mpfc_launch(H->shape64, k_coarse_solve<SCH>, dim3(1), dim3(32), coarse_smem(C), s, C, k, (const float*)H->K3[SCH - 1]);
 }
 
-// First level run by the tail kernel: the finest level of at most shape.tail_cells
+// First level run by the tail kernel: the finest level of at most sh.tail_cells
 // cells, leaving at least one level above the coarsest and at most kMaxTail levels in
 // the tail; nlev when no tail is used.
-int mpfc_tail_first_level(const mpfc_s* H) {
+int mpfc_tail_first_level(const mpfc_s* H, const mpfc_launch_shape& sh) {
   const int L = H->nlev;
-  if (H->shape.tail_cells <= 0 || L < 2) return L;
+  if (sh.tail_cells <= 0 || L < 2) return L;
   int lt = L - 1;
-  while (lt > 0 && (long long)H->lev[lt - 1].m * H->lev[lt - 1].n <= H->shape.tail_cells) --lt;
+  while (lt > 0 && (long long)H->lev[lt - 1].m * H->lev[lt - 1].n <= sh.tail_cells) --lt;
   if (lt > L - 2) return L;
   if (L - lt > kMaxTail) lt = L - kMaxTail;
   return lt;
@@ -541,7 +544,7 @@ int mpfc_tail_first_level(const mpfc_s* H) {
 // Whether a V-cycle ends with k_smooth_res on the finest level (which then runs by
 // per-level launches and has post-sweeps), so that its residual test is k_resnorm_red.
 static bool vcycle_fuses_norm(const mpfc_s* H) {
-  const int L = H->nlev, lt = mpfc_tail_first_level(H);
+  const int L = H->nlev, lt = mpfc_tail_first_level(H, H->shape64);
   const int down = lt < L ? lt : L - 1;
   return down >= 1 && H->p.nu2 >= 1;
 }
@@ -559,10 +562,10 @@ static void launch_tail(mpfc_s* H, int lt, cudaStream_t s) {
     A.lv[i].k = H->coef[SCH - 1][lt + i];
     A.lv[i].kb = H->coefb[SCH - 1][lt + i];
   }
-  const int nc = H->shape.tail_ctas;
+  const int nc = H->shape64.tail_ctas;
   const size_t smem = coarse_smem(H->lev[H->nlev - 1]);
   if (nc == 1) {   // one CTA: __syncthreads between the phases, plain (L1) loads
-    mpfc_launch(H->shape, k_tail<SCH, kLdPlain>, dim3(1), dim3(kTailThreads), smem, s, A);
+    mpfc_launch(H->shape64, k_tail<SCH, kLdPlain>, dim3(1), dim3(kTailThreads), smem, s, A);
     return;
   }
   cudaLaunchConfig_t cfg = {};
@@ -578,16 +581,16 @@ static void launch_tail(mpfc_s* H, int lt, cudaStream_t s) {
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = (nc <= H->shape.pdl_blocks) ? 2 : 1;
+  cfg.numAttrs = (nc <= H->shape64.pdl_blocks) ? 2 : 1;
   (void)cudaLaunchKernelEx(&cfg, k_tail<SCH, kLdL2>, A);
 }
 
 template <int SCH>
 static void enqueue_vcycle(mpfc_s* H, cudaStream_t s) {
   const mpfc_params& p = H->p;
-  const mpfc_launch_shape& sh = H->shape;
+  const mpfc_launch_shape& sh = H->shape64;
   const int L = H->nlev;
-  const int lt = mpfc_tail_first_level(H);
+  const int lt = mpfc_tail_first_level(H, H->shape64);
   const int down = lt < L ? lt : L - 1;   // levels smoothed and restricted by per-level launches
   for (int l = 0; l < down; ++l) {
     MpfcRange range(mpfc_level_name(l));
@@ -681,16 +684,16 @@ static void enqueue_resnorm(mpfc_s* H, int mode, cudaGraphConditionalHandle hnd,
   const Lev& L0 = H->lev[0];
   if (mode == 1 && vcycle_fuses_norm(H)) {   // after a V-cycle that ended with k_smooth_res
     int blocks = mpfc_reduce_blocks((size_t)L0.m * L0.n / 2);
-    mpfc_launch(H->shape, k_resnorm_red<SCH>, dim3(blocks), dim3(256), 0, s, L0, H->coef[SCH - 1][0], H->ctl,
+    mpfc_launch(H->shape64, k_resnorm_red<SCH>, dim3(blocks), dim3(256), 0, s, L0, H->coef[SCH - 1][0], H->ctl,
                 H->partials, (const double*)H->bpart, H->nbpart, hnd, set_cond);
     return;
   }
   int blocks = mpfc_reduce_blocks((size_t)L0.m * L0.n);
   if (mode == 0)   // right after the initial guess: rows 2 and 3 hold by construction
-    mpfc_launch(H->shape, k_resnorm<SCH, true>, dim3(blocks), dim3(256), 0, s, L0, H->coef[SCH - 1][0], H->ctl,
+    mpfc_launch(H->shape64, k_resnorm<SCH, true>, dim3(blocks), dim3(256), 0, s, L0, H->coef[SCH - 1][0], H->ctl,
                 H->partials, mode, hnd, set_cond);
   else
-    mpfc_launch(H->shape, k_resnorm<SCH>, dim3(blocks), dim3(256), 0, s, L0, H->coef[SCH - 1][0], H->ctl, H->partials,
+    mpfc_launch(H->shape64, k_resnorm<SCH>, dim3(blocks), dim3(256), 0, s, L0, H->coef[SCH - 1][0], H->ctl, H->partials,
                 mode, hnd, set_cond);
 }
 
@@ -726,7 +729,7 @@ static void learned_body(mpfc_s* H, int scheme, cudaStream_t s) {
 static void enqueue_coarse_phik(mpfc_s* H, cudaStream_t s) {
   for (int l = 1; l < H->nlev; ++l) {
     const Lev& C = H->lev[l];
-    mpfc_launch(H->shape, k_restrict_plane, grid_for(C.m, C.n, kBlk2d), kBlk2d, 0, s, (const double*)H->lev[l - 1].pk, C.pk,
+    mpfc_launch(H->shape64, k_restrict_plane, grid_for(C.m, C.n, kBlk2d), kBlk2d, 0, s, (const double*)H->lev[l - 1].pk, C.pk,
                 C.m, C.n);
   }
 }
@@ -935,14 +938,14 @@ extern "C" int mpfc_set_launch_shape(mpfc_t* H, int rows, int small_cells, int p
       tail_cells < 0 || (tail_ctas != 1 && tail_ctas != 8 && tail_ctas != 16))
     return MPFC_ERR_INVALID;
   if (tail_ctas > mpfc_tail_max_ctas()) return MPFC_ERR_INVALID;
-  H->shape = mpfc_launch_shape{rows, small_cells, pdl_blocks, tail_cells, tail_ctas, H->shape.split_cells};
+  H->shape = H->shape64 = mpfc_launch_shape{rows, small_cells, pdl_blocks, tail_cells, tail_ctas, H->shape.split_cells};
   mpfc_drop_graphs(H);
   return MPFC_OK;
 }
 
 extern "C" int mpfc_set_transfer_split(mpfc_t* H, int fine_cells) {
   if (!H || fine_cells < 0) return MPFC_ERR_INVALID;
-  H->shape.split_cells = fine_cells;
+  H->shape.split_cells = H->shape64.split_cells = fine_cells;
   mpfc_drop_graphs(H);
   return MPFC_OK;
 }
@@ -959,7 +962,7 @@ extern "C" int mpfc_launch_counts(const mpfc_t* H, int scheme, int* per_step, in
   if (!H || (scheme != 1 && scheme != 2) || H->p.precision != MPFC_FP64 || H->p.guess == MPFC_GUESS_LEARNED)
     return MPFC_ERR_INVALID;
   const mpfc_params& p = H->p;
-  const int L = H->nlev, lt = mpfc_tail_first_level(H);
+  const int L = H->nlev, lt = mpfc_tail_first_level(H, H->shape);
   const int down = lt < L ? lt : L - 1;   // levels run by per-level launches
   // per level: nu1 + nu2 sweeps of two colours, restriction, tau, prolongation
   const int per_level = 2 * p.nu1 + 2 * p.nu2 + 3;

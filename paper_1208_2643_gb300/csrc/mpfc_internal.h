@@ -92,8 +92,9 @@ struct mpfc_s {
   bool df = false;                               // the handle's V-cycles run in correction form
   cudaGraphConditionalHandle cur_handle64 = 0;   // loop of the FP64 V-cycle, for values outside the form's range
   int launch_mode = MPFC_LAUNCH_GRAPH;
-  // set by mpfc_create from the precision (mpfc_default_launch_shape)
+  // set by mpfc_create (mpfc_default_launch_shape): the step's kernels, and those of the FP64 V-cycle
   mpfc_launch_shape shape = {1, 0, 0, 0, 8};
+  mpfc_launch_shape shape64 = {1, 0, 0, 0, 8};
   // Poisson solve of the energies (poisson.cu)
   float* poisP = nullptr;               // coarsest grid's pseudo-inverse (FP32, G x G)
   cudaGraphExec_t pois_exec = nullptr;
@@ -171,7 +172,7 @@ void mpfc_build_K3(const mpfc::Lev& C, const mpfc::Coef& k, std::vector<double>&
 void mpfc_coarse_block(const mpfc::Lev& C, const mpfc::Coef& k, std::vector<float>& out);
 int mpfc_reduce_blocks(size_t G);
 int mpfc_tail_max_ctas();
-mpfc_launch_shape mpfc_default_launch_shape(int precision);
+mpfc_launch_shape mpfc_default_launch_shape(int precision, bool df);
 void mpfc_abort_capture(cudaStream_t s);
 int mpfc_capture_while(mpfc_s* H, cudaStream_t cs, cudaGraphConditionalHandle hnd,
                        void (*body_fn)(mpfc_s*, int, cudaStream_t), int scheme);
@@ -181,7 +182,7 @@ int mpfc_capture_conditional(mpfc_s* H, cudaStream_t cs, cudaGraphConditionalHan
 void mpfc_enqueue_prologue(mpfc_s* H, int scheme, cudaStream_t s);
 void mpfc_enqueue_commit(mpfc_s* H, int scheme, cudaStream_t s);
 
-int mpfc_tail_first_level(const mpfc_s* H);
+int mpfc_tail_first_level(const mpfc_s* H, const mpfc_launch_shape& sh);
 
 // correction form of the FP64 V-cycle (df_cycle.cu)
 size_t mpfc_df_carve(mpfc_s* H, const mpfc_params* p, size_t* off, char* base, const mpfc::Lev* lev,

@@ -348,7 +348,7 @@ int mpfc_pois_init(mpfc_s* H) {
   std::vector<float> P((size_t)G * G);
   for (int r = 0; r < G; ++r)
     for (int c = 0; c < G; ++c) P[(size_t)r * G + c] = (float)(A[(size_t)r * W + G + c] - 1.0 / G);
-  H->pshape = mpfc_default_launch_shape(MPFC_FP32_INNER);
+  H->pshape = mpfc_default_launch_shape(MPFC_FP32_INNER, false);
   cudaError_t e = cudaFuncSetAttribute(k_pois_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(H->poisP, P.data(), P.size() * sizeof(float), cudaMemcpyHostToDevice, H->stream);
