@@ -42,7 +42,8 @@ extern "C" {
  * of relative error 2^-46 leaves the converged step at the FP64 rounding level.  Values outside
  * the range that form covers (|phi| >= 2^20, a residual >= 2^40 or below 2^-56 and still above
  * tol) continue with FP64 V-cycles, and handles with a single level or stencil coefficients
- * outside [2^-60, 2^60] (h far below 1e-4) use those alone. */
+ * outside [2^-60, 2^60] (h far below 1e-4), and those too large for the device with the form's
+ * planes (mpfc_workspace_bytes), use those alone. */
 #define MPFC_FP64 0
 #define MPFC_FP32_INNER 1 /* FP64 outer defect correction around FP32 inner V-cycles       */
 
@@ -119,7 +120,9 @@ typedef struct mpfc_s mpfc_t;
 void mpfc_default_params(mpfc_params* p);
 
 /* Workspace bytes a handle with these parameters needs (0 if the parameters are
- * invalid).  The workspace must be device memory aligned to 256 bytes. */
+ * invalid).  The workspace must be device memory aligned to 256 bytes.  FP64 handles (and
+ * batches) whose workspace with the planes of the correction form (see MPFC_FP64) would exceed
+ * seven eighths of the current device's memory do without them. */
 size_t mpfc_workspace_bytes(const mpfc_params* p);
 
 /* Creates a solver handle on `cuda_stream` (a cudaStream_t; NULL = legacy stream).

@@ -655,7 +655,8 @@ size_t max_items(const std::vector<mpfc_params>& each, int coarsest) {
   return n + 64;
 }
 
-size_t carve_batch(mpfc_batch_s* B, int count, const mpfc_params* each, char* base) {
+// df: with the planes of the correction form.
+size_t carve_batch(mpfc_batch_s* B, int count, const mpfc_params* each, char* base, bool df) {
   BCarver c{base, 0};
   int GL = 0;
   std::vector<int> nl(count);
@@ -762,7 +763,7 @@ size_t carve_batch(mpfc_batch_s* B, int count, const mpfc_params* each, char* ba
         }
         d.pb = reinterpret_cast<float2*>(planes[6]);
         d.pk = reinterpret_cast<float2*>(planes[7]);
-      } else if (nl[i] > 1) {
+      } else if (df) {
         for (int q = 0; q < 3; ++q) d.d[q] = c.take<float2>(G);
         for (int q = 0; q < 3; ++q) d.r[q] = c.take<float2>(G);
         d.pb = c.take<float2>(G);
@@ -984,14 +985,23 @@ int build_batch_graph(mpfc_batch_s* B) {
   return MPFC_OK;
 }
 
-// The levels' coefficients, whether the batch runs in correction form (every instance has at
-// least two levels and coefficients in its range), and its tail: the last levels of every
+// The workspace's size, and whether the batch runs in correction form (every instance has at least
+// two levels and coefficients in its range, and the planes fit).
+size_t batch_layout(int count, const mpfc_params* each, bool& df) {
+  df = true;
+  for (int i = 0; i < count && df; ++i) df = mpfc_df_usable(&each[i]);
+  const size_t need = carve_batch(nullptr, count, each, nullptr, df);
+  if (!df || mpfc_df_fits(need)) return need;
+  df = false;
+  return carve_batch(nullptr, count, each, nullptr, false);
+}
+
+// The levels' coefficients and the correction form's tail: the last levels of every
 // instance, of at most kTailCells cells each, in one CTA per instance (as many as all instances
 // have).  A step of 16 instances (128^2 to 1024^2): 5.20 ms, against 5.26 with tails from 16^2
 // and 5.41 with the coarsest solve alone (FP64 V-cycles: 8.59).
 constexpr int kTailCells = 32 * 32;
 int plan_df(mpfc_batch_s* B, std::vector<DPar> (&pars)[2]) {
-  B->df = true;
   B->tail = kDfTailMax;
   for (int s = 0; s < 2; ++s) {
     B->coef[s].assign((size_t)B->count * kMaxLevels, Coef{});
@@ -1000,7 +1010,6 @@ int plan_df(mpfc_batch_s* B, std::vector<DPar> (&pars)[2]) {
     pars[s].assign((size_t)B->count * kMaxLevels, zero);
   }
   for (int i = 0; i < B->count; ++i) {
-    B->df = B->df && B->nlev[i] >= 2;
     int t = 1;
     while (t < B->nlev[i]) {
       const Lev& L = B->lev[(size_t)i * kMaxLevels + B->nlev[i] - 1 - t];
@@ -1012,7 +1021,6 @@ int plan_df(mpfc_batch_s* B, std::vector<DPar> (&pars)[2]) {
       for (int l = 0; l < B->nlev[i]; ++l) {
         const size_t id = (size_t)i * kMaxLevels + l;
         B->coef[s][id] = mpfc_coef(&B->each[i], s + 1, B->lev[id].h, 4);
-        B->df = B->df && df_coef_ok(B->coef[s][id]);
         pars[s][id].L = B->dlev[id];
         pars[s][id].k = pars[s][id].kb = df_coef_of(B->coef[s][id], s + 1, B->coef[s][id]);
       }
@@ -1053,7 +1061,8 @@ extern "C" size_t mpfc_batch_workspace_bytes(int count, const mpfc_params* each)
         each[i].guess == MPFC_GUESS_LEARNED || each[i].bc != MPFC_BC_PERIODIC || each[i].pinning)
       return 0;
   }
-  return carve_batch(nullptr, count, each, nullptr);
+  bool df;
+  return batch_layout(count, each, df);
 }
 
 extern "C" int mpfc_batch_create(int count, const mpfc_params* each, void* d_workspace, size_t bytes,
@@ -1069,8 +1078,8 @@ extern "C" int mpfc_batch_create(int count, const mpfc_params* each, void* d_wor
   B->p0 = each[0];
   B->stream = (cudaStream_t)cuda_stream;
   B->ws = (char*)d_workspace;
-  B->ws_need = need;
-  carve_batch(B, count, each, (char*)d_workspace);
+  B->ws_need = batch_layout(count, each, B->df);
+  carve_batch(B, count, each, (char*)d_workspace, B->df);
   int rc = MPFC_OK;
   do {
     cudaError_t e;

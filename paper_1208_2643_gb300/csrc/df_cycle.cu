@@ -334,20 +334,35 @@ void defect(mpfc_s* H, int mode, cudaGraphConditionalHandle hnd, int set_cond, c
 // The correction form runs on FP64 handles with at least two levels and coefficients far
 // inside the binary32 range (h = 1e-6 gives (4/h^2)(4 theta/h^2) = 1e25; the FP64 V-cycle
 // keeps such handles).
-bool mpfc_df_usable(const mpfc_s* H) {
-  if (H->p.precision != MPFC_FP64 || H->nlev < 2) return false;
-  for (int s = 0; s < 2; ++s)
-    for (int l = 0; l < H->nlev; ++l)
-      if (!df_coef_ok(H->coef[s][l]) || !df_coef_ok(H->coefb[s][l])) return false;
+bool mpfc_df_usable(const mpfc_params* p) {
+  const int L = mpfc_num_levels(p->m, p->n, p->coarsest);
+  if (p->precision != MPFC_FP64 || L < 2) return false;
+  double h = p->h;
+  for (int l = 0; l < L; ++l, h *= 2.0)
+    for (int s = 1; s <= 2; ++s)
+      if (!df_coef_ok(mpfc_coef(p, s, h, 4)) || !df_coef_ok(mpfc_coef(p, s, h, 3))) return false;
   return true;
+}
+
+// Whether a workspace with the correction form's planes (a third to two thirds more than without)
+// leaves the device room for the fields a caller keeps beside it, three planes of about twenty;
+// handles and batches too large for that keep the FP64 V-cycle and its smaller workspace.  Asked
+// of the device's whole memory, so that the size and the handle made with it agree.
+bool mpfc_df_fits(size_t workspace) {
+  if (workspace < ((size_t)8 << 30)) return true;
+  size_t free_bytes = 0, total = 0;
+  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {   // no device: the size alone is asked for
+    (void)cudaGetLastError();
+    return true;
+  }
+  return workspace <= total / 8 * 7;
 }
 
 // Planes of the correction form.  Level 0: corrections and rho in dr0, p0 and phi^k in the
 // Poisson planes (used only by mpfc_energy); coarser levels in the FP64 V-cycle's planes, which
 // it writes before it reads them, and a one-launch way up's result in planes of its own.
-size_t mpfc_df_carve(mpfc_s* H, const mpfc_params* p, size_t* off, char* base, const Lev* lev, double* const* dr0,
+size_t mpfc_df_carve(mpfc_s* H, size_t* off, char* base, const Lev* lev, double* const* dr0,
                      double* px0, double* pf0, int nlev) {
-  if (p->precision != MPFC_FP64 || nlev < 2) return 0;
   const size_t start = *off;
   auto take = [&](size_t cells) -> float2* {
     float2* q = base ? reinterpret_cast<float2*>(base + *off) : nullptr;
@@ -388,7 +403,7 @@ size_t mpfc_df_carve(mpfc_s* H, const mpfc_params* p, size_t* off, char* base, c
 }
 
 int mpfc_df_init(mpfc_s* H) {
-  if (!mpfc_df_usable(H)) return MPFC_OK;
+  if (!H->df) return MPFC_OK;
   cudaError_t e = cudaSuccess;
   auto raise = [&](auto* k) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDfTailSmem);

@@ -191,8 +191,9 @@ struct Carver {
 // scaled residual near 7e-7) still leaves three, so only those steps gain a cycle.
 constexpr double kGuessGateTolMultiple = 2.6e4;
 
-// Walks the layout; with base == nullptr only computes the size.
-static size_t carve(mpfc_s* H, const mpfc_params* p, char* base) {
+// Walks the layout; with base == nullptr only computes the size.  dfp: with the planes of the
+// correction form.
+static size_t carve(mpfc_s* H, const mpfc_params* p, char* base, bool dfp) {
   Carver c{base, 0};
   int L = mpfc_num_levels(p->m, p->n, p->coarsest);
   size_t G0 = (size_t)p->m * p->n;
@@ -212,7 +213,6 @@ static size_t carve(mpfc_s* H, const mpfc_params* p, char* base) {
   // The finest level's d and rho of the correction form; the coarse levels' planes that are dead
   // while it runs (kept R kappa_f and phi^k of the FP64 V-cycle, the energies' Poisson planes)
   // share their memory.
-  const bool dfp = p->precision == MPFC_FP64 && L >= 2;
   double* dr0[6] = {};
   const size_t dr_off = c.off;
   if (dfp)
@@ -259,7 +259,7 @@ static size_t carve(mpfc_s* H, const mpfc_params* p, char* base) {
   float* K3b = c.take<float>(2 * (size_t)Gc * Gc);
   float* poisP = c.take<float>((size_t)Gc * Gc);
   mpfc_fp32_carve(H, p, &c.off, base, L);
-  mpfc_df_carve(H, p, &c.off, base, lev, dr0, px[0], pf[0], L);
+  if (dfp) mpfc_df_carve(H, &c.off, base, lev, dr0, px[0], pf[0], L);
   mpfc_guess_carve(H, p, &c.off, base);
   if (H && base) {
     H->nlev = L;
@@ -286,9 +286,19 @@ static size_t carve(mpfc_s* H, const mpfc_params* p, char* base) {
   return c.off;
 }
 
+// The workspace's size, and whether the handle's V-cycles run in correction form.
+static size_t layout(const mpfc_params* p, bool& dfp) {
+  dfp = mpfc_df_usable(p);
+  const size_t need = carve(nullptr, p, nullptr, dfp);
+  if (!dfp || mpfc_df_fits(need)) return need;
+  dfp = false;
+  return carve(nullptr, p, nullptr, false);
+}
+
 extern "C" size_t mpfc_workspace_bytes(const mpfc_params* p) {
   if (!params_valid(p)) return 0;
-  return carve(nullptr, p, nullptr);
+  bool dfp;
+  return layout(p, dfp);
 }
 
 // K3 = I - c theta L^3 on the coarsest grid (dense, row-major G x G).
@@ -372,7 +382,8 @@ extern "C" int mpfc_create(const mpfc_params* p, void* d_workspace, size_t bytes
   if (!out) return MPFC_ERR_INVALID;
   *out = nullptr;
   if (!params_valid(p)) return MPFC_ERR_INVALID;
-  size_t need = carve(nullptr, p, nullptr);
+  bool dfp;
+  const size_t need = layout(p, dfp);
   if (!d_workspace || bytes < need || ((uintptr_t)d_workspace & 255)) return MPFC_ERR_WORKSPACE;
   mpfc_s* H = new mpfc_s();
   H->p = *p;
@@ -380,13 +391,13 @@ extern "C" int mpfc_create(const mpfc_params* p, void* d_workspace, size_t bytes
   H->stream = (cudaStream_t)cuda_stream;
   H->ws = (char*)d_workspace;
   H->ws_bytes = bytes;
-  carve(H, p, (char*)d_workspace);
+  carve(H, p, (char*)d_workspace, dfp);
   for (int s = 0; s < 2; ++s)
     for (int l = 0; l < H->nlev; ++l) {
       H->coef[s][l] = mpfc_coef(p, s + 1, H->lev[l].h, 4);
       H->coefb[s][l] = mpfc_coef(p, s + 1, H->lev[l].h, 3);
     }
-  H->df = mpfc_df_usable(H);
+  H->df = dfp;
   H->shape = mpfc_default_launch_shape(p->precision, H->df);
   H->shape64 = mpfc_default_launch_shape(p->precision, false);
   int rc = MPFC_OK;

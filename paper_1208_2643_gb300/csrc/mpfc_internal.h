@@ -185,9 +185,10 @@ void mpfc_enqueue_commit(mpfc_s* H, int scheme, cudaStream_t s);
 int mpfc_tail_first_level(const mpfc_s* H, const mpfc_launch_shape& sh);
 
 // correction form of the FP64 V-cycle (df_cycle.cu)
-size_t mpfc_df_carve(mpfc_s* H, const mpfc_params* p, size_t* off, char* base, const mpfc::Lev* lev,
+size_t mpfc_df_carve(mpfc_s* H, size_t* off, char* base, const mpfc::Lev* lev,
                      double* const* dr0, double* px0, double* pf0, int nlev);
-bool mpfc_df_usable(const mpfc_s* H);
+bool mpfc_df_usable(const mpfc_params* p);
+bool mpfc_df_fits(size_t workspace);
 int mpfc_df_init(mpfc_s* H);
 void mpfc_df_restrict_pk(mpfc_s* H, int l, cudaStream_t s);
 void mpfc_df_vcycle(mpfc_s* H, int scheme, cudaStream_t s);
