@@ -24,6 +24,7 @@ namespace mpfc {
 constexpr int kLegTile = 16;
 constexpr int kLegThreads = 288;   // 24 x 24 staged cells (nu = 2) in two passes, 22 x 22 / 2 in one
 constexpr int kLegMaxNu = 3;
+constexpr int kLegCellsPerThread = ((kLegTile + 4 * kLegMaxNu) * (kLegTile + 4 * kLegMaxNu) + kLegThreads - 1) / kLegThreads;
 
 // The staged cells' planes and (way up) the coarse correction under them with a ring.
 inline size_t leg_smem(int nu, int scheme, bool pinned, bool up) {
@@ -48,6 +49,8 @@ template <int SCH, bool NY>
 struct Leg {
   DPar P;         // the tile with its halo as a level of its own, in shared memory
   int x0, y0, ylo, W, rows;
+  int go[kLegCellsPerThread];                // where this thread's staged cells are in the level's planes,
+  int wg[kLegCellsPerThread], ws[kLegCellsPerThread];   // in the pinning weight and in its staged copy
 
   // Staged cell t (colour-split order) and its domain coordinates.
   __device__ __forceinline__ void cell(const DLev& F, int t, int& x, int& y) const {
@@ -88,14 +91,34 @@ struct Leg {
     if (!(NY && F.L.nyn)) ylo = (ylo % n + n) % n;
   }
 
+  // The offsets of the copies (integer divisions), before the wait for the previous kernel: four
+  // steps at 512^2 in 2.86 ms, 2.92 with them after it.
+  __device__ __forceinline__ void plan(const DLev& F) {
+    const int half = W >> 1, hc = half * rows;
+#pragma unroll
+    for (int q = 0; q < kLegCellsPerThread; ++q) {
+      const int t = threadIdx.x + q * kLegThreads;
+      go[q] = wg[q] = ws[q] = 0;
+      if (t >= 2 * hc) continue;
+      int x, y;
+      cell(F, t, x, y);
+      go[q] = (int)dindex(F, x, y);
+      if (SCH == 2 && F.W) {
+        const int color = t >= hc, r = (t - color * hc) / half, i = 2 * (t - color * hc - r * half) + ((r + color) & 1);
+        wg[q] = y * F.m + x;
+        ws[q] = r * W + i;
+      }
+    }
+  }
   // Starts the copies of the planes a sweep reads only, and (OWN) of d.
   template <bool OWN>
   __device__ __forceinline__ void load(const DLev& F) const {
-    const int half = W >> 1, hc = half * rows;
-    for (int t = threadIdx.x; t < 2 * hc; t += blockDim.x) {
-      int x, y;
-      cell(F, t, x, y);
-      const size_t g = dindex(F, x, y);
+    const int cells = W * rows;
+#pragma unroll
+    for (int q = 0; q < kLegCellsPerThread; ++q) {
+      const int t = threadIdx.x + q * kLegThreads;
+      if (t >= cells) continue;
+      const int g = go[q];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         leg_copy8(P.L.r[c] + t, F.r[c] + g);
@@ -104,10 +127,7 @@ struct Leg {
       leg_copy8(P.L.pb + t, F.pb + g);
       if (SCH == 2) {
         leg_copy8(P.L.pk + t, F.pk + g);
-        if (F.W) {
-          const int color = t >= hc, r = (t - color * hc) / half, i = 2 * (t - color * hc - r * half) + ((r + color) & 1);
-          leg_copy8(const_cast<double*>(P.L.W) + r * W + i, F.W + (size_t)y * F.m + x);
-        }
+        if (F.W) leg_copy8(const_cast<double*>(P.L.W) + ws[q], F.W + wg[q]);
       }
     }
   }
@@ -136,6 +156,7 @@ __global__ void __launch_bounds__(kLegThreads) k_df_down(const __grid_constant__
   extern __shared__ float2 lsm[];
   Leg<SCH, NY> T;
   T.init(F, nu, lsm);
+  T.plan(F.L);
   pdl_enter();
   T.template load<false>(F.L);
   const int half = T.W >> 1, red = half * T.rows;
@@ -176,8 +197,6 @@ __global__ void __launch_bounds__(kLegThreads) k_df_down(const __grid_constant__
   }
 }
 
-// The level's rho, p0 and d were written before the previous launch, whose start waited for them:
-// they are read before the wait for the coarse level's correction.
 template <int SCH, bool NY>
 __global__ void __launch_bounds__(kLegThreads) k_df_up(const __grid_constant__ DPar C, const __grid_constant__ DPar F,
                                                        const __grid_constant__ LegOut O, int nu) {
@@ -185,19 +204,23 @@ __global__ void __launch_bounds__(kLegThreads) k_df_up(const __grid_constant__ D
   Leg<SCH, NY> T;
   T.init(F, nu, lsm);
   const int half = T.W >> 1, hc = half * T.rows, cw = half + 2, ch = (T.rows >> 1) + 2;
-  T.template load<true>(F.L);
-  pdl_enter();
-  // the coarse correction under the staged cells with one ring
+  T.plan(F.L);
+  // the coarse correction under the staged cells with one ring, a cell a thread
+  static_assert(((kLegTile + 4 * kLegMaxNu) / 2 + 2) * ((kLegTile + 4 * kLegMaxNu) / 2 + 2) <= kLegThreads, "");
   float2* const e = lsm + (7 + (SCH == 2 ? 1 + (F.L.W != nullptr) : 0)) * 2 * hc;
-  for (int t = threadIdx.x; t < cw * ch; t += blockDim.x) {
-    const int cj = t / cw, I = (T.x0 / 2 - 1 + t - cj * cw + C.L.m) % C.L.m;
+  int ge = -1;
+  if (threadIdx.x < cw * ch) {
+    const int cj = threadIdx.x / cw, I = (T.x0 / 2 - 1 + (int)threadIdx.x - cj * cw + C.L.m) % C.L.m;
     int J = T.ylo / 2 - 1 + cj;
     if (NY && C.L.nyn) J = min(max(J, 0), C.L.n - 1);
     else J = (J + C.L.n) % C.L.n;
-    const size_t g = dindex(C.L, I, J);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) leg_copy8(e + c * cw * ch + t, C.L.d[c] + g);
+    ge = (int)dindex(C.L, I, J);
   }
+  pdl_enter();
+  T.template load<true>(F.L);
+  if (ge >= 0)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) leg_copy8(e + c * cw * ch + threadIdx.x, C.L.d[c] + ge);
   leg_copies_done();
   __syncthreads();
   for (int t = threadIdx.x; t < 2 * hc; t += blockDim.x) {

@@ -1013,16 +1013,14 @@ __global__ void __launch_bounds__(leg32_threads<T>()) k_leg32_down(Lev32 F, Lev3
   }
 }
 
-// r, q and the second copy of e were written before the previous launch, whose start waited for
-// them: they are read before the wait for the coarse level's correction.
 template <int T>
 __global__ void __launch_bounds__(leg32_threads<T>()) k_leg32_up(Lev32 C, Lev32 F, Coef32 kf, Coef32 kb, int nu) {
   constexpr int H = 4;
   extern __shared__ __align__(16) float l32[];
   Leg32<T, H, H> G;
   G.init(F, l32);
-  G.template load<true>(F, F.xphi, F.xmu, F.xka);
   pdl_enter();
+  G.template load<true>(F, F.xphi, F.xmu, F.xka);
   constexpr int cw = G.W / 2 + 2, CP = cw * (G.R / 2 + 2);
   float* const e = l32 + 7 * G.P;   // the coarse correction under the staged cells with one ring
   for (int t = threadIdx.x; t < cw * (G.S.n / 2 + 2); t += blockDim.x) {

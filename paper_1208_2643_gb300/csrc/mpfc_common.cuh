@@ -125,7 +125,10 @@ __device__ __forceinline__ double rcp_nr(double x) {
 // its memory operations are visible; launch_dependents then lets the launch of the
 // next kernel begin while this one runs, so launch latency overlaps execution instead
 // of adding to it.  For a kernel launched without the attribute both are no-ops.
-// Every kernel of the time step calls this before its first memory access.
+// Every kernel of the time step calls this before its first access to memory that a kernel of
+// the step writes (what is written once at creation may be read before it).  The order of the
+// two matters: with the signal after the wait, the kernels before the previous one have completed
+// when a kernel starts, so that its writes cannot meet their reads.
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
