@@ -253,7 +253,6 @@ __device__ __forceinline__ df df_sum_out(const float2* f, const DBlk& b) {
   return norm(addu(sum4u(ldd(f + b.out[0]), ldd(f + b.out[1]), ldd(f + b.out[2]), ldd(f + b.out[3])),
                    sum4u(ldd(f + b.out[4]), ldd(f + b.out[5]), ldd(f + b.out[6]), ldd(f + b.out[7]))));
 }
-__device__ __forceinline__ df mul2(df a, float k) { return scale2(a, k); }
 
 // Restriction at coarse cell (I, J): rho_c = R r and p0_c = R(p0 + d_phi).  The block sum of
 // the five-point Laplacian is (sum of the 8 bordering cells - 2 sum of the block) / h^2, as in

@@ -45,7 +45,6 @@ __device__ __forceinline__ df addu(df a, df b) {
   two_sum(a.h, b.h, s, e);
   return df{s, fadd(e, fadd(a.l, b.l))};
 }
-__device__ __forceinline__ df subu(df a, df b) { return addu(a, neg(b)); }
 __device__ __forceinline__ df add(df a, df b) { return norm(addu(a, b)); }
 // Sums of three and four terms, normalised once.
 __device__ __forceinline__ df sum3u(df a, df b, df c) {

@@ -31,29 +31,23 @@ constexpr int kPoisThreads = 1024;
 __device__ __forceinline__ df third() { return df{0.333333343f, -9.934108e-09f}; }
 
 // A cell's update, d <- (sum of its real neighbours + F) / (their number).
-template <int MODE>
 __device__ __forceinline__ void pois_cell(const DLev& L, int color, int x, int j, double* u = nullptr,
                                           const double* scale = nullptr) {
   const size_t own = (color ? dplane(L) : 0) + (size_t)j * (L.m >> 1) + x;
-  const df F = ldd(L.r[0] + own);
-  df s = F;
   const bool edge = L.nyn && (j == 0 || j == L.n - 1);
-  if (MODE != kAll) {
-    const DNb o = df_nb<true>(L, color, x, j, own);
-    auto at = [&](size_t q) { return q == own ? df{0.f, 0.f} : ldd(L.d[0] + q); };   // a ghost is the cell itself
-    s = addu(norm(sum4u(ldd(L.d[0] + o.c0), ldd(L.d[0] + o.cx), at(o.s), at(o.n))), F);
-  }
+  const DNb o = df_nb<true>(L, color, x, j, own);
+  auto at = [&](size_t q) { return q == own ? df{0.f, 0.f} : ldd(L.d[0] + q); };   // a ghost is the cell itself
+  const df s = addu(norm(sum4u(ldd(L.d[0] + o.c0), ldd(L.d[0] + o.cx), at(o.s), at(o.n))), ldd(L.r[0] + own));
   const df d = edge ? mul(norm(s), third()) : scale2(norm(s), 0.25f);
   L.d[0][own] = f2(d);
   if (u) u[(size_t)j * L.m + 2 * x + ((j + color) & 1)] += df_to_f64(d) * *scale;   // a power of two: exact
 }
 
-template <int MODE>
 __global__ void __launch_bounds__(256) k_pois_half(const __grid_constant__ DLev L, int color, double* u, const double* scale) {
   pdl_enter();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= (L.m >> 1) || j >= L.n) return;
-  pois_cell<MODE>(L, color, x, j, u, scale);
+  pois_cell(L, color, x, j, u, scale);
 }
 
 // F_c = sum over the block of F + sum_nb d - 4 d, and the coarse level's first red half sweep.
@@ -120,10 +114,9 @@ struct PoisTail {
   DLev lv[kPoisTailMax];
 };
 
-template <int MODE>
 __device__ __forceinline__ void pois_tail_half(const DLev& L, int color) {
   const int half = L.m >> 1, cells = half * L.n;
-  for (int t = threadIdx.x; t < cells; t += blockDim.x) pois_cell<MODE>(L, color, t % half, t / half);
+  for (int t = threadIdx.x; t < cells; t += blockDim.x) pois_cell(L, color, t % half, t / half);
   __syncthreads();
 }
 
@@ -156,9 +149,9 @@ __global__ void __launch_bounds__(kPoisThreads) k_pois_tail(const __grid_constan
   for (int l = 0; l < A.nlev - 1; ++l) {
     const DLev& F = sl[l];
     const DLev& C = sl[l + 1];
-    pois_tail_half<kGen>(F, 1);
-    pois_tail_half<kGen>(F, 0);
-    pois_tail_half<kGen>(F, 1);
+    pois_tail_half(F, 1);
+    pois_tail_half(F, 0);
+    pois_tail_half(F, 1);
     const int cc = C.m * C.n;
     for (int t = tid; t < cc; t += nt) pois_restrict_cell(F, C, t % C.m, t / C.m);
     __syncthreads();
@@ -172,7 +165,7 @@ __global__ void __launch_bounds__(kPoisThreads) k_pois_tail(const __grid_constan
     for (int t = tid; t < cc; t += nt) df_prolong_plane(C, F, 0, t % C.m, t / C.m);
     __syncthreads();
     for (int sw = 0; sw < 2; ++sw)
-      for (int color = 0; color < 2; ++color) pois_tail_half<kGen>(F, color);
+      for (int color = 0; color < 2; ++color) pois_tail_half(F, color);
   }
   for (int t = tid; t < G; t += nt) g.d[0][t] = sl[0].d[0][t];
 }
@@ -275,7 +268,7 @@ size_t pois_tail_smem(const mpfc_s* H, int lt) {
 
 void pois_half(const mpfc_s* H, const DLev& L, int color, double* u, cudaStream_t s) {
   const mpfc_launch_shape& sh = H->pshape;
-  mpfc_launch(sh, k_pois_half<kGen>, mpfc_grid_of(sh, L.m / 2, L.n), mpfc_blk_for(sh, L.m / 2, L.n), 0, s, L, color, u,
+  mpfc_launch(sh, k_pois_half, mpfc_grid_of(sh, L.m / 2, L.n), mpfc_blk_for(sh, L.m / 2, L.n), 0, s, L, color, u,
               (const double*)&H->ctl->sums[4]);
 }
 
