@@ -34,7 +34,11 @@ if ROOT not in sys.path:
 METRIC = "MPFC steps/s & cell-updates/s at 1024^2: plain FAS vs learned/FP32/batched, tol 1e-10"
 UNIT = "steps/s"
 
-# Algorithmic FP64 flops of one red-black sweep per cell (scheme 1, relaxed update):
+# Instructions of one cell update of the correction form's half sweep (scheme 1): ncu's
+# smsp__inst_executed.sum of k_df_smooth at 1024^2 times 32 lanes over its 2^19 cells
+# (profiles/launches_correction_form_1024.md).
+DF_SMOOTH_INSTR_PER_CELL = 536
+# Algorithmic FP64 flops of one red-black sweep of the FP64 V-cycle per cell (scheme 1, relaxed update):
 # neighbour sums 9, right-hand sides 7, Newton terms of the cubic 5, determinant 2,
 # reciprocal 1, Cramer numerators 9, phi/mu products 2, kappa 2, relaxation 9.
 SMOOTH_FLOPS_PER_CELL = 46
@@ -211,6 +215,14 @@ def cpu_oracle_rate(size, scheme, max_steps, budget_s, warmup=0, threaded=False)
             break
     dt = time.perf_counter() - t0
     return done / dt, done, dt, cycles, nthreads
+
+
+def issue_peak(clk):
+    """Warp instructions per second of this GPU: four sub-partitions an SM, one a cycle, at the
+    median SM clock under load (the maximum where no sample was taken)."""
+    import torch
+    mhz = clk.get("sm_mhz") or clk.get("sm_max_mhz") or 2070.0
+    return 4.0 * torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count * mhz * 1e6
 
 
 # ----------------------------------------------------------------------------- reference arm
@@ -407,7 +419,17 @@ def run_ours(args):
             print(json.dumps({"profile_run": True, "ms": ms, "cycles": cycles[:5]}), flush=True)
         return
 
-    # dominant kernel: the finest-level red-black sweep, timed on the solver's stream
+    # dominant kernel: the finest level's red-black sweep in float-float, timed through the batch's
+    # sweep timer on one instance (the cell function of the step's k_df_smooth, two launches)
+    from paper_1208_2643_gb300 import tuning
+    one = mpfc.BatchSolver([p], stream=stream)
+    one.set_state(0, phi0)
+    tuning.autotune(one, scheme, reps=2)
+    df_sweep_ms = one.time_smooth(scheme, 0, reps=50)
+    one.close()
+    df_winstr = DF_SMOOTH_INSTR_PER_CELL * size * size / 32.0 / (df_sweep_ms * 1e-3)
+
+    # the FP64 V-cycle's sweep (steps outside the correction form's range), on the solver's stream
     phik, _, _ = solver.get_state(device=True)
     S = solver.op_source(scheme, phik, phik, torch.zeros_like(phik))
     u = [phik.clone(), torch.zeros_like(phik), torch.zeros_like(phik)]
@@ -500,9 +522,10 @@ def run_ours(args):
     for obj in (s32, a64, a32):
         obj.close()
     # the FP32 sweep against the HBM roofline, at 2048^2 (the mixed-precision workload's size,
-    # planes 7 x 16 MB): after an L2 flush, one pair of red-black sweeps as the inner cycles
-    # run them at that size (one launch per sweep over shared-memory tiles, there and back
-    # between the two copies of e), per sweep = half the pair; median of 7.  Beside it the
+    # planes 7 x 16 MB), as mpfc_set_fp32_sweep selects it (by default a level's sweeps are part of
+    # its one-launch ways): after an L2 flush, one pair of red-black sweeps in one launch each
+    # over shared-memory tiles, there and back between the two copies of e, per sweep = half the
+    # pair; median of 7.  Beside it the
     # two-launch sweep (one launch per colour, in place).  40 algorithmic bytes per cell (e
     # read and written, r and q read).
     if rank == 0:
@@ -524,7 +547,7 @@ def run_ours(args):
         gbs2 = 40.0 * 2048 * 2048 / (us_two * 1e-6) / 1e9
         forms["fp32_inner"]["sweep_roofline"] = {
             "kernel": "k_sweep32_tiles<16>, one red+black sweep at 2048^2 (half of a there-and-back pair after an "
-                      "L2 flush)", "us": us_tiled,
+                      "L2 flush; selected by mpfc_set_fp32_sweep, not launched by default)", "us": us_tiled,
             "bound": "hbm", "achieved_gbs": gbs, "peak_gbs": peaks["hbm_gbs"], "frac": gbs / peaks["hbm_gbs"],
             "peak_source": ("MEASURED_PEAKS.json hbm_gbs (of measured)" if peaks["source"] == "measured"
                             else "6.8 TB/s, an earlier GB300 measurement (of fallback)"),
@@ -603,8 +626,10 @@ def run_ours(args):
                                     "vcycles_per_instance_step": float(np.mean(cy64)) / 2, "steps": 2,
                                     "smooth_sweep": {"kernel": "kb_df_half<1>, one red+black sweep of the 64 finest "
                                                               "levels in float-float (two launches)",
-                                                    "ms": ms_kb, "bound": "fp32 issue",
-                                                    "cell_updates_per_s": kb_cells}}
+                                                    "ms": ms_kb, "cell_updates_per_s": kb_cells,
+                                                    "bound": "instruction issue and memory",
+                                                    "frac_of_issue": DF_SMOOTH_INSTR_PER_CELL * kb_cells / 32.0 /
+                                                    issue_peak(clk)}}
         b64.close()
 
     # learned initial guess (model trained by paper_1208_2643_gb300.guess on solver data at 256^2)
@@ -841,15 +866,26 @@ def run_ours(args):
                 "vcycles_per_step": float(np.mean(cycles)) if cycles else None,
                 "sweep_cell_updates_per_s": steps_per_s * size * size * (p.nu1 + p.nu2) *
                 (float(np.mean(cycles)) if cycles else 0.0),
-                "roofline": {"bound": "alu", "kernel": "k_smooth<1> (finest level, one red+black sweep; the FP64 V-cycle's, which the "
-                                       "step takes outside the correction form's range)",
-                             "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s (FP64, FMA = 2)",
-                             "frac": achieved / fp64_peak,
-                             "peak_source": "measured live: FP64 FMA-chain probe on this GPU",
-                             "hbm_gbs_algorithmic": achieved_gbs,
-                             "sweep_ms": sweep_ms,
-                             "traffic": traffic_for("k_smooth", size),
-                             "steady_state": steady},
+                "roofline": {"bound": "instruction issue",
+                             "kernel": "kb_df_half<1> on one instance: one red+black sweep of the finest level in "
+                                       "float-float (the cell function of k_df_smooth, which leads the step), back to "
+                                       "back, planes in L2",
+                             "achieved": df_winstr / 1e9, "peak": issue_peak(clk) / 1e9, "unit": "G warp instructions/s",
+                             "frac": df_winstr / issue_peak(clk),
+                             "peak_source": "one instruction a cycle and sub-partition at the median SM clock of the "
+                                            "timed region",
+                             "sweep_ms": df_sweep_ms, "instructions_per_cell": DF_SMOOTH_INSTR_PER_CELL, "traffic": None},
+                "roofline_fp64_cycle": {"bound": "alu",
+                                        "kernel": "k_smooth<1>, one red+black sweep of the finest level in FP64 (not "
+                                                  "launched by the timed steps: the FP64 V-cycle runs outside the "
+                                                  "correction form's range)",
+                                        "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s (FP64, FMA = 2)",
+                                        "frac": achieved / fp64_peak,
+                                        "peak_source": "measured live: FP64 FMA-chain probe on this GPU",
+                                        "hbm_gbs_algorithmic": achieved_gbs,
+                                        "sweep_ms": sweep_ms,
+                                        "traffic": traffic_for("k_smooth", size),
+                                        "steady_state": steady},
                 "forms": forms,
                 "e2e": e2e, "gpu_launches": launches, "clocks": clk, "cpu_baseline": cpu}
         print(json.dumps(line), flush=True)
