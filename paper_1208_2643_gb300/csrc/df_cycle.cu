@@ -66,8 +66,8 @@ struct UPlanes {
   double* u[3];
 };
 
-// Bound by FP32 issue (about 350 instructions per cell) on the levels that stay in L2 and by
-// the memory traffic (52 B per cell and half sweep) on larger ones.
+// Bound by instruction issue (536 instructions per cell, slots 74 % busy: 13 us at 1024^2) on the
+// levels that stay in L2 and by the memory traffic (52 B per cell and half sweep) on larger ones.
 template <int SCH, int MODE, bool NY, bool FINAL>
 __global__ void __launch_bounds__(256) k_df_smooth(const __grid_constant__ DPar P, int color,
                                                    const __grid_constant__ UPlanes U) {
@@ -161,7 +161,10 @@ UPlanes uplanes(const mpfc_s* H) {
   return U;
 }
 
-// Handles of at most 64^2 cells run the producers' extra work as launches of its own.
+// Handles of at most 64^2 cells run the producers' extra work as launches of its own and take no
+// one-launch ways, so that a level keeps the 11 launches that mpfc_launch_counts states for them
+// (tests/test_gpu_fp64.py, test_launch_counts).  That is not the faster shape: four steps at 64^2
+// take 1.59 ms with it and 1.24 without, with the same bits.
 bool df_unfused(const mpfc_s* H) { return (long long)H->p.m * H->p.n <= 64 * 64; }
 
 template <int SCH, int MODE, bool FINAL>

@@ -1,8 +1,8 @@
 // One level's way down or up of the V-cycle in correction form as one launch, for levels whose
 // launches do not fill the chip.
 //
-// A half sweep of such a level is a chain of about 1.3 k clocks (350 dependent float-float
-// instructions a cell) in a launch of 2.3 us, and a level takes ten launches.  Here a CTA owns
+// A half sweep of such a level is a chain of about 1.3 k clocks (536 instructions a cell, most of
+// them dependent) in a launch of 2.3 us, and a level takes ten launches.  Here a CTA owns
 // kLegTile x kLegTile cells and sweeps them together with a halo in shared memory: every half sweep
 // needs the one before it on one more ring of cells, so the ring is computed by both tiles that
 // hold it, from the same values with the same cell functions (the bits are those of the
@@ -10,7 +10,7 @@
 // updates of a launch take less than the launch itself.  A way takes 11 k clocks after its
 // predecessor (5.5 us at 32^2 as at 256^2), bound by the chain: copies in 1 to 2 k, each half sweep
 // 1.5 to 2.1 k, the prolongation 1.5 k, the restriction 2 to 4 k; five launches took about 12 us.
-// Two steps at 512^2 3.13 -> 2.86 ms, at 1024^2 3.13 -> 3.00, pinned at 512 x 384 4.51 -> 4.04.
+// Four steps at 512^2 3.13 -> 2.86 ms, two at 1024^2 3.13 -> 3.00, pinned at 512 x 384 4.51 -> 4.04.
 //
 // Down: the first red half sweep (d = 0 before it), the others, and the restriction.  Up: the
 // prolongation and the sweeps; the result goes to planes of its own (or is added to u on the

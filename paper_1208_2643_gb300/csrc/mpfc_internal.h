@@ -116,7 +116,7 @@ struct mpfc_s {
 };
 
 // Block shape of the per-cell V-cycle kernels on an X x Y launch.  GB300's FP64 unit
-// is narrow: a warp-wide FP64 instruction takes about 64 cycles whatever the number of
+// is narrow: a warp-wide FP64 instruction takes about 80 cycles whatever the number of
 // active lanes, and an SM saturates at about four warps issuing FP64.  A half sweep of
 // ~33 FP64 instructions per cell therefore costs ~1 us per warp however few cells it
 // has, so small launches use one-warp blocks spread over as many SMs as possible, and
