@@ -39,9 +39,9 @@ extern "C" {
 /* MPFC_FP64: FP64 iterate, source, residual, convergence test and state.  The V-cycle works on
  * the change it makes to the iterate (correction form of the FAS cycle: the same iterates in
  * exact arithmetic), carried in float-float numbers (48 bits) from an FP64 residual.  An
- * operation rounds by 2^-44 to 2^-46 of its operands, and one cycle's iterate was measured up to
- * 8e-13 off (40 times an FP64 cycle's; mpfc_step_cycles shows it); the next cycle's FP64 residual
- * takes that up, so a converged step is at the FP64 rounding level.  Values outside
+ * operation rounds by 2^-44 to 2^-46 of its operands, and the iterate after one cycle was measured
+ * 2e-13 to 5e-12 off, 10 to 120 times an FP64 cycle's (mpfc_step_cycles shows it); the next cycles'
+ * FP64 residuals take that up, so a converged step is at the FP64 rounding level.  Values outside
  * the range that form covers (|phi| >= 2^20, a residual >= 2^40 or below 2^-56 and still above
  * tol) continue with FP64 V-cycles, and handles with a single level or stencil coefficients
  * outside [2^-60, 2^60] (h far below 1e-4), and those too large for the device with the form's
